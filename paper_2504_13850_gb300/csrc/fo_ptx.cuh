@@ -83,6 +83,17 @@ __device__ __forceinline__ void tma_4d(void* dst, const CUtensorMap* m, uint64_t
       "l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(bar)), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
       : "memory");
 }
+// im2col-mode load: pixels in (n, h, w) order over the map's bounding box from
+// the one at (w, h, n), shifted by the tap offset (ow, oh) from its lower corner.
+__device__ __forceinline__ void tma_im2col(void* dst, const CUtensorMap* m, uint64_t* bar, int c, int w, int h, int n,
+                                           int ow, int oh) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.im2col.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], "
+      "[%2], {%7, %8};" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(bar)), "r"(c), "r"(w), "r"(h), "r"(n), "h"(uint16_t(ow)),
+      "h"(uint16_t(oh))
+      : "memory");
+}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 

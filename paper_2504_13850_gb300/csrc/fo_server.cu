@@ -1074,6 +1074,12 @@ int build_plan(fo_server* s) {
   return FO_OK;
 }
 
+// Bytes of a tensor's buffer: room for the images its im2col map declares.
+int64_t im2col_room(const Tensor& t) {
+  const int64_t image = int64_t(t.bytes()) / t.N;
+  return t.dt == fo::kBF16 ? fo::im2col_images(t.N, image) * image : int64_t(t.bytes());
+}
+
 int allocate(fo_server* s) {
   const fo_server_cfg& c = s->cfg;
   size_t esz = s->dt == fo::kF32 ? 4 : 2;
@@ -1093,10 +1099,16 @@ int allocate(fo_server* s) {
   // activation slab: omega slots (Eq. 3), 256-byte aligned each
   s->slot_act_bytes = int64_t(c.batch) * c.in_h * c.in_w * c.in_c * esz;
   s->slot_stride = (s->slot_act_bytes + 255) / 256 * 256;
+  // a slot that a convolution window reads is long enough for its im2col map
+  if (s->dt == fo::kBF16)
+    for (const fo_op& op : s->ops)
+      if (op.kind == FO_OP_CONV && s->T[op.in0].is_input() && (op.k > 1 || op.stride > 1))
+        s->slot_stride = std::max(s->slot_stride, (im2col_room(s->T[0]) + 255) / 256 * 256);
   s->slab = (char*)s->alloc(size_t(s->slot_stride) * c.omega);
   s->slot_labels = (int32_t*)s->alloc(size_t(c.omega) * c.batch * 4);
   s->slot_lengths = (int32_t*)s->alloc(size_t(c.omega) * c.batch * 4);
   if (!s->slab || !s->slot_labels || !s->slot_lengths) return set_err(FO_ERR_OOM, "activation slab");
+  FO_CUDA(cudaMemset(s->slab, 0, size_t(s->slot_stride) * c.omega));
   s->slot_ready.assign(c.omega, nullptr);
   s->slot_free.assign(c.omega, nullptr);
   s->slot_consumed.assign(c.omega, 0);
@@ -1120,9 +1132,14 @@ int allocate(fo_server* s) {
   for (int tid = 1; tid <= nops; ++tid) {
     Tensor& t = s->T[tid];
     if (t.root != tid) continue;
-    t.act = s->alloc(t.bytes());
-    t.grad = s->alloc(t.bytes());
+    const size_t room = size_t(im2col_room(t));   // zero past the tensor
+    t.act = s->alloc(room);
+    t.grad = s->alloc(room);
     if (!t.act || !t.grad) return set_err(FO_ERR_OOM, "tensor allocation");
+    if (room > t.bytes()) {
+      FO_CUDA(cudaMemset(t.act, 0, room));
+      FO_CUDA(cudaMemset(t.grad, 0, room));
+    }
   }
   for (int tid = 1; tid <= nops; ++tid) {
     Tensor& t = s->T[tid];

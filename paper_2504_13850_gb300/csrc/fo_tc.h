@@ -15,6 +15,15 @@ namespace fo {
 struct TcContext;
 struct TcGemm;
 
+// im2col tensor maps never describe a tensor shorter than this: a shorter one
+// is declared with more images, so the buffers they read (activations and
+// their gradients, and batch slots) have room for these, zero past the tensor.
+constexpr int64_t kIm2colMinBytes = 128 * 1024;
+inline int64_t im2col_images(int64_t n, int64_t image_bytes) {
+  const int64_t least = (kIm2colMinBytes + image_bytes - 1) / image_bytes;
+  return n > least ? n : least;
+}
+
 int tc_create(TcContext** out, fo_server* s);
 void tc_destroy(TcContext* c);
 // Selects the tensor maps of batch slot `slot` for the first layer.

@@ -20,7 +20,7 @@ namespace {
 // The epilogue variant a plan's parameters ask for.
 int epi_of(const TcParams& p) {
   return (p.out_f32 ? E_F32 : 0) | (p.relu ? E_RELU : 0) | (p.mask ? E_MASK : 0) | (p.acc ? E_ACC : 0) |
-         (p.pool_out ? E_POOL : 0) | (p.tma_out ? E_TMA : 0) | (p.gelu_out ? E_GELU : 0);
+         (p.pool_out ? E_POOL : 0) | (p.tma_out ? E_TMA : 0) | (p.gelu_out ? E_GELU : 0) | (p.im2col ? E_I2C : 0);
 }
 
 KernelFn pick_kernel(int kind, int bn, bool cluster, int epi, size_t* smem) {
@@ -43,16 +43,25 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+typedef CUresult (*EncodeIm2colFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                   const cuuint64_t*, const int*, const int*, cuuint32_t, cuuint32_t,
+                                   const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+void* driver_entry(const char* name) {
+  void* p = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  if (cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+      q == cudaDriverEntryPointSuccess)
+    return p;
+  return nullptr;
+}
 EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-  }
+  static EncodeTiledFn fn = reinterpret_cast<EncodeTiledFn>(driver_entry("cuTensorMapEncodeTiled"));
+  return fn;
+}
+EncodeIm2colFn encode_im2col_fn() {
+  static EncodeIm2colFn fn = reinterpret_cast<EncodeIm2colFn>(driver_entry("cuTensorMapEncodeIm2col"));
   return fn;
 }
 
@@ -120,6 +129,29 @@ bool map_window_chunked(CUtensorMap* m, const void* base, int N, int H, int W, i
   uint32_t elem[5] = {1, uint32_t(stride), uint32_t(stride), 1, 1};
   return make_map(m, base, 5, dims, strides, box, elem);
 }
+// im2col-mode map over the same tensor: a load takes `pixels` positions in
+// (n, h, w) order out of a bounding box that starts at `lo` (rows and columns
+// alike) and ends `hi_h` rows / `hi_w` columns past the tensor's last ones
+// (negative: before them), stepping `stride`, 64 channels each; the tap offset
+// comes with the load, and positions outside the tensor read zero.  A short
+// tensor is declared with more (zero) images, see im2col_images; their pixels
+// only reach GEMM rows that are not stored or meet zero rows of the other
+// operand.
+bool map_im2col(CUtensorMap* m, const void* base, int N, int H, int W, int C, int lo, int hi_h, int hi_w, int stride,
+                int pixels) {
+  EncodeIm2colFn fn = encode_im2col_fn();
+  const int64_t img = int64_t(H) * W * C * 2;
+  // corners are signed bytes
+  if (!fn || C % 64 || lo < -128 || hi_h < -128 || hi_w < -128 || hi_h > 127 || hi_w > 127) return false;
+  const int64_t images = im2col_images(N, img);
+  cuuint64_t dims[4] = {cuuint64_t(C), cuuint64_t(W), cuuint64_t(H), cuuint64_t(images)};
+  cuuint64_t strides[3] = {cuuint64_t(C) * 2, cuuint64_t(W) * C * 2, cuuint64_t(img)};
+  const int lower[2] = {lo, lo}, upper[2] = {hi_w, hi_h};
+  cuuint32_t elem[4] = {1, cuuint32_t(stride), cuuint32_t(stride), 1};
+  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, lower, upper, 64,
+            cuuint32_t(pixels), elem, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 bool map_window(CUtensorMap* m, const void* base, int N, int H, int W, int C, int ow, int rows, int imgs,
                 int stride = 1) {
   uint64_t dims[4] = {uint64_t(C), uint64_t(W), uint64_t(H), uint64_t(N)};
@@ -163,9 +195,9 @@ struct TcContext {
 
 namespace {
 
-bool window_ok(int N, int H, int W, int rows_needed, int* rows, int* imgs) {
-  // A box of `rows_needed` pixels made of whole image rows (and whole images
-  // when it spans several).
+// A box of `rows_needed` pixels made of whole image rows (and whole images
+// when it spans several); images past the last one read as zero.
+bool window_ok(int H, int W, int rows_needed, int* rows, int* imgs) {
   if (W > 256 || rows_needed % W) return false;
   int r = rows_needed / W;
   if (r <= H) {
@@ -178,15 +210,23 @@ bool window_ok(int N, int H, int W, int rows_needed, int* rows, int* imgs) {
     *imgs = r / H;
     if (*imgs > 256) return false;
   }
-  (void)N;
   return true;
+}
+// A strided convolution's tiled boxes need every output to own a whole
+// stride x stride patch of the input.  Where either rule fails (7, 14 or 28
+// pixel rows, odd maps) the window is loaded in im2col mode; such layers ran
+// on the CUDA-core kernel before (bf16, 5-9 TFLOP/s against 200-240 here):
+// ResNet-18 stages 3-4 on 28 x 28 maps at batch 24, 20.6 -> 0.72 ms a step;
+// the VGG part at batch 37, whose last tile is partial, 8.0 -> 0.26 ms.
+bool whole_windows(const fo_op& op, const Tensor& a, const Tensor& o) {
+  return op.stride == 1 || (a.H == 2 * o.H && a.W == 2 * o.W);
 }
 
 
 // Split-K clusters of S CTAs of kernel (kind, bn) that fit on the GPU at
 // once (GPC packing), from the occupancy calculator; cached per context.
 int active_clusters(TcContext* c, int kind, int bn, int S, int epi) {
-  const int key = ((kind * 512 + bn) * 16 + S) * 16 + epi;
+  const int key = ((kind * 512 + bn) * 16 + S) * 256 + epi;
   auto it = c->cluster_fit.find(key);
   if (it != c->cluster_fit.end()) return it->second;
   size_t smem = 0;
@@ -247,7 +287,7 @@ void choose_tiles(TcContext* c, TcGemm* g, int M, int N, int KB, int ndiv) {
     const double stage_kb = (BM + bn) * BK * 2 / 1024.0;
     const double epi = bn == 256 ? 4.2 : (bn == 128 ? 2.2 : 1.5);
     double t_kb = std::max(0.37, stage_kb / 128.0);
-    if (win_b) t_kb = std::max(t_kb, 0.39);
+    if (win_b) t_kb = std::max(t_kb, g->p.im2col ? 0.1 + 0.1 * bn / 64 : 0.39);   // im2col: one box per 64 channels
     for (int sp = 1; sp <= 8; ++sp) {
       if (sp > 1 && KB / sp < 4) break;
       // an owner's receive slices (16 KB per other rank and owned chunk) live in the pipeline buffers
@@ -418,7 +458,7 @@ TcGemm* tc_plan_forward(TcContext* c, fo_server* s, int i, void* out, bool relu,
     return nullptr;
   if (ex && ex->pool_out) {   // whole 2 x 2 windows inside each warp's 32 rows
     const bool w_ok = o.W == 2 || o.W == 4 || o.W == 8 || o.W == 16;
-    if (!relu || !w_ok || o.H % 2 || o.C % 8 || o.rows() % BM) return nullptr;
+    if (!relu || !w_ok || o.H % 2 || o.C % 8 || o.rows() % 32) return nullptr;
   }
   TcGemm* g = new TcGemm();
   g->p.out = out;
@@ -446,25 +486,31 @@ TcGemm* tc_plan_forward(TcContext* c, fo_server* s, int i, void* out, bool relu,
   }
   // convolution: k in {1, 3}, stride in {1, 2}; tiles of 128 output pixels
   const int st = op.stride, Ho = o.H, Wo = o.W;
-  if (op.cin % 64 || op.cout % 64 || (st == 2 && (a.H != 2 * Ho || a.W != 2 * Wo))) { delete g; return nullptr; }
+  if (op.cin % 64 || op.cout % 64) { delete g; return nullptr; }
   int rows, imgs;
-  if (!window_ok(a.N, Ho, Wo, BM, &rows, &imgs) || (int64_t(a.N) * Ho * Wo) % BM) { delete g; return nullptr; }
+  const bool tiled = whole_windows(op, a, o) && window_ok(Ho, Wo, BM, &rows, &imgs);
+  if (ex && ex->pool_out && !tiled) { delete g; return nullptr; }
   g->kind = CONV_FPROP;
   g->name = "tc_conv_fprop";
   g->p.H = Ho; g->p.W = Wo; g->p.ksz = op.k; g->p.pad = op.k / 2; g->p.taps = op.k * op.k; g->p.stride = st;
   g->p.cblocks = op.cin / 64;
   g->p.ntap_ch = op.cin;
-  g->p.win_rows = rows; g->p.win_imgs = imgs;
+  g->p.im2col = tiled ? 0 : 1;
+  g->p.lo = -g->p.pad;
   int M = a.N * Ho * Wo, KB = g->p.taps * g->p.cblocks;
   choose_tiles(c, g, M, op.cout, KB, op.cout);
   const int bn = g->bn;
-  const int box_rows = rows, box_imgs = imgs;
+  auto map_a = [&](CUtensorMap* m, const void* base) {
+    if (tiled) return map_window(m, base, a.N, a.H, a.W, a.C, Wo, rows, imgs, st);
+    const int hi = g->p.pad - (op.k - 1);   // the last output's first tap
+    return map_im2col(m, base, a.N, a.H, a.W, a.C, -g->p.pad, hi, hi, st, BM);
+  };
   g->input_A = s->T[op.in0].is_input();
   if (g->input_A) {
     g->slot_maps.resize(s->cfg.omega);
     for (int sl = 0; sl < s->cfg.omega; ++sl)
-      if (!map_window(&g->slot_maps[sl], s->slab + size_t(sl) * s->slot_stride, a.N, a.H, a.W, a.C, Wo, box_rows, box_imgs, st)) { delete g; return nullptr; }
-  } else if (!map_window(&g->p.tmA, tensor_act(s, op.in0), a.N, a.H, a.W, a.C, Wo, box_rows, box_imgs, st)) { delete g; return nullptr; }
+      if (!map_a(&g->slot_maps[sl], s->slab + size_t(sl) * s->slot_stride)) { delete g; return nullptr; }
+  } else if (!map_a(&g->p.tmA, tensor_act(s, op.in0))) { delete g; return nullptr; }
   if (!map_2d(&g->p.tmB, w, op.cout, int64_t(g->p.taps) * op.cin, bn)) { delete g; return nullptr; }
   return finish(c, g, M, op.cout, double(g->p.taps) * op.cin);
 }
@@ -507,15 +553,17 @@ bool tc_plan_dgrad(TcContext* c, fo_server* s, int i, int accumulate, void* dx, 
   // input row y = st*i + py receives output row p = i + dh from tap r when
   // st*dh = py + pad - r.  Each class is an implicit GEMM over its own taps.
   const int st = op.stride, pad = op.k / 2, Ho = o.H, Wo = o.W;
-  if (op.cin % 64 || op.cout % 64 || (st == 2 && (a.H != 2 * Ho || a.W != 2 * Wo))) return false;
+  if (op.cin % 64 || op.cout % 64) return false;
   int rows, imgs;
-  if (!window_ok(o.N, Ho, Wo, BM, &rows, &imgs) || (int64_t(o.N) * Ho * Wo) % BM) return false;
+  const bool tiled = whole_windows(op, a, o) && window_ok(Ho, Wo, BM, &rows, &imgs);
   const int nclass = st * st;
   bool any_empty = false;
-  struct Cls { int n; int rs[9], dh[9], dw[9]; } cls[4];
+  struct Cls { int n, H, W; int rs[9], dh[9], dw[9]; } cls[4];
   for (int q = 0; q < nclass; ++q) {
     const int py = q / st, px = q % st;
     cls[q].n = 0;
+    cls[q].H = (a.H - py + st - 1) / st;   // input rows and columns of this parity
+    cls[q].W = (a.W - px + st - 1) / st;
     for (int r = 0; r < op.k; ++r)
       for (int sx = 0; sx < op.k; ++sx) {
         const int vh = py + pad - r, vw = px + pad - sx;
@@ -531,12 +579,16 @@ bool tc_plan_dgrad(TcContext* c, fo_server* s, int i, int accumulate, void* dx, 
   const int eff_acc = any_empty && !accumulate ? 1 : accumulate;
   *zero_first = any_empty && !accumulate;
   for (int q = 0; q < nclass; ++q) {
-    if (cls[q].n == 0) continue;
+    if (cls[q].n == 0 || cls[q].H == 0 || cls[q].W == 0) continue;
     TcGemm* g = base();
     g->p.acc = eff_acc;
     g->kind = CONV_DGRAD;
     g->name = "tc_conv_dgrad";
-    g->p.H = Ho; g->p.W = Wo; g->p.ksz = op.k; g->p.pad = pad; g->p.taps = op.k * op.k;
+    const int Hq = cls[q].H, Wq = cls[q].W;   // Ho x Wo when tiled
+    g->p.H = Hq; g->p.W = Wq; g->p.ksz = op.k; g->p.pad = pad; g->p.taps = op.k * op.k;
+    g->p.im2col = tiled ? 0 : 1;
+    g->p.lo = 0;
+    for (int t = 0; t < cls[q].n; ++t) g->p.lo = std::min(g->p.lo, std::min(cls[q].dh[t], cls[q].dw[t]));
     g->p.cblocks = op.cout / 64;
     g->p.ntap_ch = op.cin;
     g->p.ntap = cls[q].n;
@@ -547,14 +599,15 @@ bool tc_plan_dgrad(TcContext* c, fo_server* s, int i, int accumulate, void* dx, 
     }
     if (st == 2) {
       g->p.ostride = 2; g->p.py = q / 2; g->p.px = q % 2;
-      g->p.Hq = Ho; g->p.Wq = Wo; g->p.oH = a.H; g->p.oW = a.W;
+      g->p.Hq = Hq; g->p.Wq = Wq; g->p.oH = a.H; g->p.oW = a.W;
     }
-    const int M = o.N * Ho * Wo, KB = cls[q].n * g->p.cblocks;
+    const int M = o.N * Hq * Wq, KB = cls[q].n * g->p.cblocks;
     choose_tiles(c, g, M, op.cin, KB, op.cin);
-    if (!map_window(&g->p.tmA, o.grad, o.N, Ho, Wo, o.C, Wo, rows, imgs) ||
-        !map_2d(&g->p.tmB, w, op.cout, int64_t(g->p.taps) * op.cin, BK)) {
+    const bool mapped = tiled ? map_window(&g->p.tmA, o.grad, o.N, Ho, Wo, o.C, Wo, rows, imgs)
+                              : map_im2col(&g->p.tmA, o.grad, o.N, Ho, Wo, o.C, g->p.lo, Hq - Ho + g->p.lo,
+                                           Wq - Wo + g->p.lo, 1, BM);
+    if (!mapped || !map_2d(&g->p.tmB, w, op.cout, int64_t(g->p.taps) * op.cin, BK)) {
       delete g;
-      for (TcGemm* x : *out) (void)x;
       out->clear();
       return false;
     }
@@ -608,15 +661,19 @@ TcGemm* tc_plan_wgrad(TcContext* c, fo_server* s, int i) {
     return finish(c, g, op.cout, op.cin, double(rows));
   }
   const int st = op.stride, Ho = o.H, Wo = o.W;
-  if (op.cin % 64 || op.cout % 128 || (st == 2 && (a.H != 2 * Ho || a.W != 2 * Wo))) { delete g; return nullptr; }
+  if (op.cin % 64 || op.cout % 128) { delete g; return nullptr; }
   int rows, imgs;
-  if (!window_ok(a.N, Ho, Wo, BK, &rows, &imgs) || (int64_t(a.N) * Ho * Wo) % BK) { delete g; return nullptr; }
+  const bool tiled = whole_windows(op, a, o) && window_ok(Ho, Wo, BK, &rows, &imgs);
   g->kind = CONV_WGRAD;
   g->name = "tc_conv_wgrad";
   g->p.ldo = op.k * op.k * op.cin;
   g->p.H = Ho; g->p.W = Wo; g->p.ksz = op.k; g->p.pad = op.k / 2; g->p.taps = op.k * op.k; g->p.stride = st;
   g->p.ntap_ch = op.cin;
-  int P = a.N * Ho * Wo, KB = P / BK;
+  g->p.im2col = tiled ? 0 : 1;
+  g->p.lo = -g->p.pad;
+  // pixels past the last one: zero rows of dy (beyond its map), so whatever
+  // the window of x holds there adds nothing
+  int P = a.N * Ho * Wo, KB = (P + BK - 1) / BK;
   int N = g->p.taps * op.cin;
   choose_tiles(c, g, op.cout, N, KB, op.cin);
   g->input_B = s->T[op.in0].is_input();
@@ -624,8 +681,10 @@ TcGemm* tc_plan_wgrad(TcContext* c, fo_server* s, int i) {
   CUtensorMap ca;
   if (map_chunked(&ca, o.grad, P, op.cout, BK, BM / 64)) { g->p.tmA = ca; g->p.chunk_a = 1; }
   const int nchunk = std::min(g->bn, op.cin) / 64;   // channel chunks per box (one box per tap)
-  g->p.chunk_b = 1;
+  g->p.chunk_b = tiled ? 1 : 0;
   auto map_b = [&](CUtensorMap* m, const void* base) {
+    const int hi = g->p.pad - (op.k - 1);
+    if (!tiled) return map_im2col(m, base, a.N, a.H, a.W, a.C, -g->p.pad, hi, hi, st, BK);
     if (g->p.chunk_b && map_window_chunked(m, base, a.N, a.H, a.W, a.C, Wo, rows, imgs, st, nchunk)) return true;
     g->p.chunk_b = 0;
     return map_window(m, base, a.N, a.H, a.W, a.C, Wo, rows, imgs, st);

@@ -50,6 +50,13 @@ enum Epi : int {
                 // accumulate operand), written into tensor memory before the
                 // tile's MMAs, and each 32 x 32 chunk leaves through shared
                 // memory by a TMA tensor store (tmO)
+  E_I2C = 128,  // convolutions: the window's tensor map is in im2col mode, so that
+                // a tile is 128 (weight gradient: a k-block is 64) consecutive
+                // pixels of the H x W grid, whatever its size.  The tiled boxes of
+                // the other variants hold whole image rows and need 128 (64) pixels
+                // to be whole rows of one image or whole images; where they do,
+                // they are kept: a weight gradient brings all channel chunks of
+                // its window in one box, im2col one box per 64 channels.
 };
 
 constexpr int BM = 128;      // UMMA M (cta_group::1)
@@ -72,7 +79,8 @@ struct TcParams {
   int stride;           // CONV_FPROP / CONV_WGRAD: stride of the windowed input
   int cblocks;          // 64-channel blocks per tap (contraction channels)
   int ntap_ch;          // CONV_WGRAD / CONV_DGRAD: channels per tap in the N index (Ci)
-  int win_rows, win_imgs;  // rows/images covered by one window box
+  int im2col;           // E_I2C
+  int lo;               // E_I2C: lower corner of the bounding box, rows and columns
   // CONV_DGRAD: the taps of this output-parity class, as (tap index r*k+s,
   // row shift, column shift) of the gradient window
   int ntap;
@@ -289,7 +297,7 @@ __device__ __forceinline__ void epilogue_chunk32(const TcParams& p, uint32_t sta
     size_t prow;
     int r0;
     pool_window(p, m_base, win, &prow, &r0);
-    if (n + 8 * co < p.N) {
+    if (n + 8 * co < p.N && m_base < p.M) {   // M % 32 == 0: the warp's rows are all inside or all outside
       float best[8];
       int arg[8];
 #pragma unroll
@@ -374,8 +382,17 @@ struct KindTraits {
   static constexpr bool b_mn = (KIND == LIN_DGRAD || KIND == LIN_WGRAD || KIND == CONV_DGRAD || KIND == CONV_WGRAD);
 };
 
+// One im2col box of the pixels from `pix` on (the H x W grid of p, spacing
+// `stride` in the tensor), channels from c0, at tap offset (oh, ow) >= 0 from
+// the bounding box's lower corner.
+__device__ __forceinline__ void load_im2col(const TcParams& p, const CUtensorMap* m, void* dst, uint64_t* bar, int pix,
+                                            int stride, int c0, int oh, int ow) {
+  const int HW = p.H * p.W, n = pix / HW, rem = pix % HW;
+  tma_im2col(dst, m, bar, c0, (rem % p.W) * stride + p.lo, (rem / p.W) * stride + p.lo, n, ow, oh);
+}
+
 // Issue the TMA loads of k-block `kb` for output tile (m0, n0).
-template <int KIND, int BN>
+template <int KIND, int BN, int EPI>
 __device__ __forceinline__ void load_kblock(const TcParams& p, int kb, int m0, int n0, char* sa, char* sb,
                                             uint64_t* bar) {
   const int HW = p.H * p.W;
@@ -391,11 +408,13 @@ __device__ __forceinline__ void load_kblock(const TcParams& p, int kb, int m0, i
     const int tap = kb / p.cblocks, c0 = (kb % p.cblocks) * 64;
     const int r = tap / p.ksz, s = tap % p.ksz;
     const int n_img = m0 / HW, h0 = (m0 % HW) / p.W;   // H, W: output grid
-    tma_4d(sa, &p.tmA, bar, c0, s - p.pad, h0 * p.stride + r - p.pad, n_img);
+    if constexpr (EPI & E_I2C) load_im2col(p, &p.tmA, sa, bar, m0, p.stride, c0, r, s);
+    else tma_4d(sa, &p.tmA, bar, c0, s - p.pad, h0 * p.stride + r - p.pad, n_img);
   } else {  // CONV_DGRAD: window over the output gradient, shifted per tap
     const int t = kb / p.cblocks, c0 = (kb % p.cblocks) * 64;
-    const int n_img = m0 / HW, h0 = (m0 % HW) / p.W;   // H, W: the class grid (= gradient grid)
-    tma_4d(sa, &p.tmA, bar, c0, p.tap_dw[t], h0 + p.tap_dh[t], n_img);
+    const int n_img = m0 / HW, h0 = (m0 % HW) / p.W;   // H, W: the class grid (= gradient grid when tiled)
+    if constexpr (EPI & E_I2C) load_im2col(p, &p.tmA, sa, bar, m0, 1, c0, p.tap_dh[t] - p.lo, p.tap_dw[t] - p.lo);
+    else tma_4d(sa, &p.tmA, bar, c0, p.tap_dw[t], h0 + p.tap_dh[t], n_img);
   }
   if (KIND == LIN_FWD) {
     tma_2d(sb, &p.tmB, bar, kb * BK, n0);
@@ -416,7 +435,7 @@ __device__ __forceinline__ void load_kblock(const TcParams& p, int kb, int m0, i
     else
 #pragma unroll
       for (int j = 0; j < BN / 64; ++j) tma_2d(sb + j * BK * 128, &p.tmB, bar, tap * p.ntap_ch + n0 + j * 64, co0);
-  } else if (p.chunk_b) {  // CONV_WGRAD: the tile's channel chunks in one box per tap
+  } else if (!(EPI & E_I2C) && p.chunk_b) {  // CONV_WGRAD: the tile's channel chunks in one box per tap
     // (a tile wider than Ci spans BN / Ci taps; a ragged last tile's tap past
     // the last one loads a shifted window whose columns the epilogue drops)
     const int cw = BN < p.ntap_ch ? BN : p.ntap_ch;
@@ -436,7 +455,8 @@ __device__ __forceinline__ void load_kblock(const TcParams& p, int kb, int m0, i
       const int nn = n0 + j * 64;
       const int tap = nn / p.ntap_ch, ci = nn % p.ntap_ch;
       const int r = tap / p.ksz, s = tap % p.ksz;
-      tma_4d(sb + j * BK * 128, &p.tmB, bar, ci, s - p.pad, h0 * p.stride + r - p.pad, n_img);
+      if constexpr (EPI & E_I2C) load_im2col(p, &p.tmB, sb + j * BK * 128, bar, pix0, p.stride, ci, r, s);
+      else tma_4d(sb + j * BK * 128, &p.tmB, bar, ci, s - p.pad, h0 * p.stride + r - p.pad, n_img);
     }
   }
 }
@@ -519,7 +539,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
         if (*abort_flag) break;
         char* sa = smem + s * STAGE_BYTES;
         mbar_expect_tx(&full[s], STAGE_BYTES);
-        load_kblock<KIND, BN>(p, kb0 + it, m0, n0, sa, sa + A_BYTES, &full[s]);
+        load_kblock<KIND, BN, EPI>(p, kb0 + it, m0, n0, sa, sa + A_BYTES, &full[s]);
       }
     }
   } else if (warp == 1) {
@@ -604,7 +624,7 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
       if (c + 1 < c1) load_row32<EPI>(p, mg, n0 + 32 * (c + 1), mk2, ac2);
       uint32_t r[32];
       tmem_ld32(trow + uint32_t(32 * c), r);
-      if (mg < p.M || (EPI & E_POOL)) {   // a pooled conv has M % 128 == 0: every lane takes part
+      if (mg < p.M) {   // a pooled conv has M % 32 == 0: every lane of the warp takes part, or none
         float v[32];
 #pragma unroll
         for (int j = 0; j < 32; ++j) v[j] = 0.f;
@@ -838,7 +858,7 @@ __global__ void __launch_bounds__(kPersistThreads, 1) tc_gemm_persistent(const _
           }
           char* sa = smem + s * STAGE_BYTES;
           mbar_expect_tx(&full[s], STAGE_BYTES);
-          load_kblock<KIND, BN>(p, kb, m0, n0, sa, sa + A_BYTES, &full[s]);
+          load_kblock<KIND, BN, EPI>(p, kb, m0, n0, sa, sa + A_BYTES, &full[s]);
         }
       }
     }
