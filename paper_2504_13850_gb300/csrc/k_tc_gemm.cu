@@ -255,16 +255,15 @@ int active_clusters(TcContext* c, int kind, int bn, int S, int epi) {
 
 // Tile width and K split from a cost model in microseconds,
 // fitted to GB300 timelines of these kernels:
-//  * a k-block stage costs at least ~0.37 us: each stage is one round of
-//    mbarrier waits (full on the MMA side, empty on the TMA side), whose
-//    dependent latency is a few hundred cycles on each side;
-//  * the TMA fills one SM's shared memory at ~128 GB/s, which bounds stages
-//    of 256-wide tiles (48 KB);
-//  * a stage issues four 128 x BN x 16 MMAs, and each takes ~190 cycles
-//    whatever BN <= 256 (measured: 128- and 256-wide weight-gradient stages
-//    both ~0.38-0.40 us once all chunks of an operand come in one TMA box),
-//    so 256-wide tiles run at the measured dense bf16 rate (about 3/4 of
-//    the nominal one) and 128-wide ones at half of it: the floor above;
+//  * a k-block stage alone costs 0.204 / 0.231 / 0.345 us at widths 64 / 128
+//    / 256 (32 k-blocks a tile, every SM busy; MN-major 0.258 / 0.398 at 128 /
+//    256): narrow tiles are bounded by the round of mbarrier waits and the MMA
+//    issue of a stage, the 256-wide tile by 192 KB in flight over a TMA round
+//    trip of ~1.4 us.  In a step, narrow tiles cost the kernels beside them
+//    more L2 traffic for the same work; 0.30 / 0.32 / 0.375 gave the best
+//    whole steps (us; these / 0.37, 0.37, 0.375 / 0.21, 0.24, 0.36): VGG 270 /
+//    269 / 271, ResNet 540 / 544 / 532, ResNet on 28 x 28 maps 643 / 662 / 660,
+//    transformer 741 / 756 / 775, one narrow ragged block 269 / 278 / 289;
 //  * a CTA pays a start-up ramp and the epilogue of its last tile (earlier
 //    epilogues overlap the next tile's MMAs), a K-split cluster pays the
 //    exchange of its partial tiles through the L2 workspace and their
@@ -284,10 +283,10 @@ void choose_tiles(TcContext* c, TcGemm* g, int M, int N, int KB, int ndiv) {
     if (win_a && (ndiv % bn || N % bn)) continue;
     if (win_b && ndiv % bn && (bn % ndiv || bn > 2 * ndiv)) continue;
     const int n_tiles = (N + bn - 1) / bn, m_tiles = (M + BM - 1) / BM, tiles = n_tiles * m_tiles;
-    const double stage_kb = (BM + bn) * BK * 2 / 1024.0;
     const double epi = bn == 256 ? 4.2 : (bn == 128 ? 2.2 : 1.5);
-    double t_kb = std::max(0.37, stage_kb / 128.0);
-    if (win_b) t_kb = std::max(t_kb, g->p.im2col ? 0.1 + 0.1 * bn / 64 : 0.39);   // im2col: one box per 64 channels
+    const bool mn = g->kind == LIN_WGRAD || win_b;
+    double t_kb = (bn == 256 ? 0.375 : (bn == 128 ? 0.32 : 0.30)) + (mn ? 0.015 : 0.0);
+    if (win_b && g->p.im2col) t_kb = std::max(t_kb, 0.1 + 0.1 * bn / 64);   // one box per 64 channels
     for (int sp = 1; sp <= 8; ++sp) {
       if (sp > 1 && KB / sp < 4) break;
       // an owner's receive slices (16 KB per other rank and owned chunk) live in the pipeline buffers

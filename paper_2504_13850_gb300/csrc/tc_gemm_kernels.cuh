@@ -1,8 +1,8 @@
 // Tensor-core GEMM / implicit-GEMM convolution for sm_103a: tcgen05.mma
 // (kind::f16, bf16 operands, fp32 accumulator in TMEM) fed by TMA tiles in
 // 128-byte-swizzled shared memory, with a warp-specialised pipeline:
-//   warp 0      TMA producer (one thread)
-//   warp 1      TMEM allocator and MMA issuer (one thread)
+//   warp 0      TMA producer (one elected lane)
+//   warp 1      TMEM allocator and MMA issuer (one elected lane)
 //   epilogue    tcgen05.ld of the 128 x BN accumulator, then the bias /
 //               ReLU / ReLU mask / residual add and the bf16 or fp32 store
 //               (four warps in the split-K kernel, eight in the persistent one)
@@ -382,84 +382,155 @@ struct KindTraits {
   static constexpr bool b_mn = (KIND == LIN_DGRAD || KIND == LIN_WGRAD || KIND == CONV_DGRAD || KIND == CONV_WGRAD);
 };
 
-// One im2col box of the pixels from `pix` on (the H x W grid of p, spacing
-// `stride` in the tensor), channels from c0, at tap offset (oh, ow) >= 0 from
-// the bounding box's lower corner.
-__device__ __forceinline__ void load_im2col(const TcParams& p, const CUtensorMap* m, void* dst, uint64_t* bar, int pix,
-                                            int stride, int c0, int oh, int ow) {
-  const int HW = p.H * p.W, n = pix / HW, rem = pix % HW;
-  tma_im2col(dst, m, bar, c0, (rem % p.W) * stride + p.lo, (rem / p.W) * stride + p.lo, n, ow, oh);
+// The MMAs of one pipeline stage (operands A then B at shared address `a0`)
+// into the accumulator at `d`, added to it when `acc`, and their commit to
+// `empty`.  Called by the one lane that elect_one picked in a converged warp:
+// the compiler then knows that descriptors and addresses are uniform.  In a
+// branch on the lane number it moved each of them through a per-lane path,
+// which cost ~0.08 us a stage and bounded every tile narrower than 256 (32
+// k-blocks a tile, 152 CTAs: 0.283 -> 0.204 us a stage at BN = 64, 0.288 ->
+// 0.231 at 128 K-major, 0.292 -> 0.258 MN-major; 256 is bounded by its bytes
+// in flight, 0.345).
+template <int KIND, int BN>
+__device__ __forceinline__ void mma_stage(uint32_t d, uint32_t a0, bool acc, uint64_t* empty) {
+  constexpr bool amn = KindTraits<KIND>::a_mn, bmn = KindTraits<KIND>::b_mn;
+  constexpr uint32_t idesc = instr_desc(BN, amn, bmn);
+  const uint32_t b0 = a0 + BM * BK * 2;
+  const uint64_t ad = amn ? smem_desc(a0, BK * 128, 1024) : smem_desc(a0, 16, 1024);
+  const uint64_t bd = bmn ? smem_desc(b0, BK * 128, 1024) : smem_desc(b0, 16, 1024);
+#pragma unroll
+  for (int k = 0; k < BK / UK; ++k)   // the address field counts 16-byte units and does not overflow (227 KB)
+    mma_f16(d, ad + k * (amn ? UK * 8 : UK / 8), bd + k * (bmn ? UK * 8 : UK / 8), idesc, acc || k > 0 ? 1u : 0u);
+  mma_commit(empty);
 }
 
-// Issue the TMA loads of k-block `kb` for output tile (m0, n0).
+// The TMA loads of consecutive k-blocks of output tile (m0, n0).  The window
+// coordinates advance by additions: as divisions of the k-block index they
+// were ~300 cycles of each stage in the producer's path.
 template <int KIND, int BN, int EPI>
-__device__ __forceinline__ void load_kblock(const TcParams& p, int kb, int m0, int n0, char* sa, char* sb,
-                                            uint64_t* bar) {
-  const int HW = p.H * p.W;
-  if (KIND == LIN_FWD || KIND == LIN_DGRAD) {
-    tma_2d(sa, &p.tmA, bar, kb * BK, m0);
-  } else if (KIND == LIN_WGRAD || KIND == CONV_WGRAD) {
-    if (p.chunk_a)
-      tma_3d(sa, &p.tmA, bar, 0, kb * BK, m0 / 64);
-    else
-#pragma unroll
-      for (int j = 0; j < BM / 64; ++j) tma_2d(sa + j * BK * 128, &p.tmA, bar, m0 + j * 64, kb * BK);
-  } else if (KIND == CONV_FPROP) {  // windowed A over the (strided) input
-    const int tap = kb / p.cblocks, c0 = (kb % p.cblocks) * 64;
-    const int r = tap / p.ksz, s = tap % p.ksz;
-    const int n_img = m0 / HW, h0 = (m0 % HW) / p.W;   // H, W: output grid
-    if constexpr (EPI & E_I2C) load_im2col(p, &p.tmA, sa, bar, m0, p.stride, c0, r, s);
-    else tma_4d(sa, &p.tmA, bar, c0, s - p.pad, h0 * p.stride + r - p.pad, n_img);
-  } else {  // CONV_DGRAD: window over the output gradient, shifted per tap
-    const int t = kb / p.cblocks, c0 = (kb % p.cblocks) * 64;
-    const int n_img = m0 / HW, h0 = (m0 % HW) / p.W;   // H, W: the class grid (= gradient grid when tiled)
-    if constexpr (EPI & E_I2C) load_im2col(p, &p.tmA, sa, bar, m0, 1, c0, p.tap_dh[t] - p.lo, p.tap_dw[t] - p.lo);
-    else tma_4d(sa, &p.tmA, bar, c0, p.tap_dw[t], h0 + p.tap_dh[t], n_img);
-  }
-  if (KIND == LIN_FWD) {
-    tma_2d(sb, &p.tmB, bar, kb * BK, n0);
-  } else if (KIND == CONV_FPROP) {
-    const int tap = kb / p.cblocks, c0 = (kb % p.cblocks) * 64;
-    tma_2d(sb, &p.tmB, bar, tap * p.ntap_ch + c0, n0);
-  } else if (KIND == LIN_DGRAD || KIND == LIN_WGRAD) {
-    if (p.chunk_b)
-      tma_3d(sb, &p.tmB, bar, 0, kb * BK, n0 / 64);
-    else
-#pragma unroll
-      for (int j = 0; j < BN / 64; ++j) tma_2d(sb + j * BK * 128, &p.tmB, bar, n0 + j * 64, kb * BK);
-  } else if (KIND == CONV_DGRAD) {
-    const int t = kb / p.cblocks, co0 = (kb % p.cblocks) * 64;
-    const int tap = p.tap_rs[t];
-    if (p.chunk_b)
-      tma_3d(sb, &p.tmB, bar, 0, co0, (tap * p.ntap_ch + n0) / 64);
-    else
-#pragma unroll
-      for (int j = 0; j < BN / 64; ++j) tma_2d(sb + j * BK * 128, &p.tmB, bar, tap * p.ntap_ch + n0 + j * 64, co0);
-  } else if (!(EPI & E_I2C) && p.chunk_b) {  // CONV_WGRAD: the tile's channel chunks in one box per tap
-    // (a tile wider than Ci spans BN / Ci taps; a ragged last tile's tap past
-    // the last one loads a shifted window whose columns the epilogue drops)
-    const int cw = BN < p.ntap_ch ? BN : p.ntap_ch;
-    const int pix0 = kb * BK;
-    const int n_img = pix0 / HW, h0 = (pix0 % HW) / p.W;
-    for (int t = 0; t * cw < BN; ++t) {
-      const int nn = n0 + t * cw;
-      const int tap = nn / p.ntap_ch, ci0 = nn % p.ntap_ch;
-      const int r = tap / p.ksz, s = tap % p.ksz;
-      tma_5d(sb + t * (cw / 64) * BK * 128, &p.tmB, bar, 0, s - p.pad, h0 * p.stride + r - p.pad, n_img, ci0 / 64);
+struct KLoader {
+  static constexpr bool kWin = KIND == CONV_FPROP || KIND == CONV_DGRAD;
+  static constexpr bool kI2c = (EPI & E_I2C) != 0;
+  static constexpr int NB = BN / 64;
+  int m0, n0, k0;          // k0: first contraction index of the k-block
+  int n, h, w;             // window kinds: image and grid position of the first pixel
+  int c0, r, s;            // fprop / dgrad: channel; fprop: tap row, column; dgrad: r = tap of the class
+  int dn, dh, dw;          // weight gradient: advance of (n, h, w) by BK pixels
+  int br[NB], bs[NB], bc[NB];   // weight gradient: tap and channel of each box
+
+  __device__ __forceinline__ void init(const TcParams& p, int m0_, int n0_, int kb) {
+    m0 = m0_;
+    n0 = n0_;
+    k0 = kb * BK;
+    if constexpr (kWin || KIND == CONV_WGRAD) {
+      const int HW = p.H * p.W, pix = kWin ? m0 : k0, rem = pix % HW;
+      n = pix / HW;
+      h = rem / p.W;
+      w = rem % p.W;
     }
-  } else {  // CONV_WGRAD: N index = tap * Ci + ci; K = output pixel
-    const int pix0 = kb * BK;
-    const int n_img = pix0 / HW, h0 = (pix0 % HW) / p.W;   // H, W: output grid
+    if constexpr (kWin) {
+      const int t = kb / p.cblocks;
+      c0 = (kb % p.cblocks) * 64;
+      r = KIND == CONV_FPROP ? t / p.ksz : t;
+      s = KIND == CONV_FPROP ? t % p.ksz : 0;
+    }
+    if constexpr (KIND == CONV_WGRAD) {   // N index = tap * Ci + ci; K = output pixel
+      const int HW = p.H * p.W, rem = BK % HW;
+      dn = BK / HW;
+      dh = rem / p.W;
+      dw = rem % p.W;
+      const int cw = !kI2c && p.chunk_b ? (BN < p.ntap_ch ? BN : p.ntap_ch) : 64;
 #pragma unroll
-    for (int j = 0; j < BN / 64; ++j) {
-      const int nn = n0 + j * 64;
-      const int tap = nn / p.ntap_ch, ci = nn % p.ntap_ch;
-      const int r = tap / p.ksz, s = tap % p.ksz;
-      if constexpr (EPI & E_I2C) load_im2col(p, &p.tmB, sb + j * BK * 128, bar, pix0, p.stride, ci, r, s);
-      else tma_4d(sb + j * BK * 128, &p.tmB, bar, ci, s - p.pad, h0 * p.stride + r - p.pad, n_img);
+      for (int j = 0; j < NB; ++j) {
+        const int nn = n0 + j * cw, tap = nn / p.ntap_ch;
+        bc[j] = nn % p.ntap_ch;
+        br[j] = tap / p.ksz;
+        bs[j] = tap % p.ksz;
+      }
     }
   }
-}
+  __device__ __forceinline__ void next(const TcParams& p) {
+    k0 += BK;
+    if constexpr (kWin) {
+      c0 += 64;
+      if (c0 == p.cblocks * 64) {
+        c0 = 0;
+        if (KIND == CONV_DGRAD) {
+          ++r;
+        } else if (++s == p.ksz) {
+          s = 0;
+          ++r;
+        }
+      }
+    }
+    if constexpr (KIND == CONV_WGRAD) {
+      w += dw;
+      h += dh;
+      n += dn;
+      if (w >= p.W) {
+        w -= p.W;
+        ++h;
+      }
+      if (h >= p.H) {
+        h -= p.H;
+        ++n;
+      }
+    }
+  }
+  // the tap offset of an im2col load counts from the bounding box's lower corner
+  __device__ __forceinline__ void im2col(const TcParams& p, const CUtensorMap* m, void* dst, uint64_t* bar, int stride,
+                                         int c, int oh, int ow) const {
+    tma_im2col(dst, m, bar, c, w * stride + p.lo, h * stride + p.lo, n, ow, oh);
+  }
+  __device__ __forceinline__ void load(const TcParams& p, char* sa, char* sb, uint64_t* bar) const {
+    if constexpr (KIND == LIN_FWD || KIND == LIN_DGRAD) {
+      tma_2d(sa, &p.tmA, bar, k0, m0);
+    } else if constexpr (KIND == LIN_WGRAD || KIND == CONV_WGRAD) {
+      if (p.chunk_a)
+        tma_3d(sa, &p.tmA, bar, 0, k0, m0 / 64);
+      else
+#pragma unroll
+        for (int j = 0; j < BM / 64; ++j) tma_2d(sa + j * BK * 128, &p.tmA, bar, m0 + j * 64, k0);
+    } else if constexpr (KIND == CONV_FPROP) {  // windowed A over the (strided) input; H, W: output grid
+      if constexpr (kI2c) im2col(p, &p.tmA, sa, bar, p.stride, c0, r, s);
+      else tma_4d(sa, &p.tmA, bar, c0, s - p.pad, h * p.stride + r - p.pad, n);
+    } else {  // CONV_DGRAD: window over the output gradient, shifted per tap; H, W: the class grid
+      if constexpr (kI2c) im2col(p, &p.tmA, sa, bar, 1, c0, p.tap_dh[r] - p.lo, p.tap_dw[r] - p.lo);
+      else tma_4d(sa, &p.tmA, bar, c0, p.tap_dw[r], h + p.tap_dh[r], n);
+    }
+    if constexpr (KIND == LIN_FWD || KIND == CONV_FPROP) {   // W's columns are the k-blocks in order (tap, channel)
+      tma_2d(sb, &p.tmB, bar, k0, n0);
+    } else if constexpr (KIND == LIN_DGRAD || KIND == LIN_WGRAD) {
+      if (p.chunk_b)
+        tma_3d(sb, &p.tmB, bar, 0, k0, n0 / 64);
+      else
+#pragma unroll
+        for (int j = 0; j < NB; ++j) tma_2d(sb + j * BK * 128, &p.tmB, bar, n0 + j * 64, k0);
+    } else if constexpr (KIND == CONV_DGRAD) {
+      const int col = p.tap_rs[r] * p.ntap_ch + n0;
+      if (p.chunk_b)
+        tma_3d(sb, &p.tmB, bar, 0, c0, col / 64);
+      else
+#pragma unroll
+        for (int j = 0; j < NB; ++j) tma_2d(sb + j * BK * 128, &p.tmB, bar, col + j * 64, c0);
+    } else if (!kI2c && p.chunk_b) {  // CONV_WGRAD: the tile's channel chunks in one box per tap
+      // (a tile wider than Ci spans BN / Ci taps; a ragged last tile's tap past
+      // the last one loads a shifted window whose columns the epilogue drops)
+      const int cw = BN < p.ntap_ch ? BN : p.ntap_ch;
+#pragma unroll
+      for (int t = 0; t < NB; ++t)
+        if (t * cw < BN)
+          tma_5d(sb + t * (cw / 64) * BK * 128, &p.tmB, bar, 0, bs[t] - p.pad, h * p.stride + br[t] - p.pad, n,
+                 bc[t] / 64);
+    } else {
+#pragma unroll
+      for (int j = 0; j < NB; ++j) {
+        if constexpr (kI2c) im2col(p, &p.tmB, sb + j * BK * 128, bar, p.stride, bc[j], br[j], bs[j]);
+        else tma_4d(sb + j * BK * 128, &p.tmB, bar, bc[j], bs[j] - p.pad, h * p.stride + br[j] - p.pad, n);
+      }
+    }
+  }
+};
 
 // Split-K: the gridDim.z CTAs of a (1, 1, S) cluster each run k-blocks
 // [kb0, kb0 + kper) of the same output tile.  Rank z owns the 32-column
@@ -528,46 +599,36 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
   pdl_wait();      // the previous kernel's writes are visible from here on
 
   if (warp == 0) {
-    if (lane == 0) {
-      for (int it = 0; it < nk; ++it) {
-        const int s = it % STAGES;
-        if (!mbar_wait(&empty[s], ((it / STAGES) & 1) ^ 1)) {
-          atomicExch(p.err, 1);
-          *abort_flag = 1;
-          break;
-        }
-        if (*abort_flag) break;
+    KLoader<KIND, BN, EPI> ld;
+    ld.init(p, m0, n0, kb0);
+    for (int it = 0; it < nk; ++it, ld.next(p)) {
+      const int s = it % STAGES;
+      if (!mbar_wait(&empty[s], ((it / STAGES) & 1) ^ 1)) {
+        atomicExch(p.err, 1);
+        *abort_flag = 1;
+        break;
+      }
+      if (*abort_flag) break;
+      if (elect_one()) {
         char* sa = smem + s * STAGE_BYTES;
         mbar_expect_tx(&full[s], STAGE_BYTES);
-        load_kblock<KIND, BN, EPI>(p, kb0 + it, m0, n0, sa, sa + A_BYTES, &full[s]);
+        ld.load(p, sa, sa + A_BYTES, &full[s]);
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = instr_desc(BN, KindTraits<KIND>::a_mn, KindTraits<KIND>::b_mn);
-      bool ok = true;
-      for (int it = 0; it < nk; ++it) {
-        const int s = it % STAGES;
-        if (!mbar_wait(&full[s], (it / STAGES) & 1)) {
-          atomicExch(p.err, 2);
-          *abort_flag = 1;
-          ok = false;
-          break;
-        }
-        tc_fence_after();
-        const uint32_t a0 = smem_u32(smem + s * STAGE_BYTES);
-        const uint32_t b0 = a0 + A_BYTES;
-#pragma unroll
-        for (int k = 0; k < BK / UK; ++k) {
-          uint64_t ad, bd;
-          if (KindTraits<KIND>::a_mn) ad = smem_desc(a0 + k * UK * 128, BK * 128, 1024);
-          else ad = smem_desc(a0 + k * UK * 2, 16, 1024);
-          if (KindTraits<KIND>::b_mn) bd = smem_desc(b0 + k * UK * 128, BK * 128, 1024);
-          else bd = smem_desc(b0 + k * UK * 2, 16, 1024);
-          mma_f16(tmem, ad, bd, idesc, (it > 0 || k > 0) ? 1u : 0u);
-        }
-        mma_commit(&empty[s]);
+    bool ok = true;
+    for (int it = 0; it < nk; ++it) {
+      const int s = it % STAGES;
+      if (!mbar_wait(&full[s], (it / STAGES) & 1)) {
+        atomicExch(p.err, 2);
+        *abort_flag = 1;
+        ok = false;
+        break;
       }
+      tc_fence_after();
+      if (elect_one()) mma_stage<KIND, BN>(tmem, smem_u32(smem + s * STAGE_BYTES), it > 0, &empty[s]);
+    }
+    if (elect_one()) {
       if (ok) mma_commit(accum);
       else mbar_expect_tx(accum, 0);  // release the epilogue without data
     }
@@ -845,68 +906,56 @@ __global__ void __launch_bounds__(kPersistThreads, 1) tc_gemm_persistent(const _
   pdl_wait();
 
   if (warp == 0) {
-    if (lane == 0) {
-      uint32_t g = 0;
-      for (int t = unit; t < tiles && !*abort_flag; t += units) {
-        const int n0 = tile_n0(t), m0 = tile_m0(t);
-        for (int kb = 0; kb < KB; ++kb, ++g) {
-          const int s = g % STAGES;
-          if (!mbar_wait(&empty[s], ((g / STAGES) & 1) ^ 1)) {
-            atomicExch(p.err, 4);
-            *abort_flag = 1;
-            break;
-          }
+    uint32_t g = 0;
+    for (int t = unit; t < tiles && !*abort_flag; t += units) {
+      KLoader<KIND, BN, EPI> ld;
+      ld.init(p, tile_m0(t), tile_n0(t), 0);
+      for (int kb = 0; kb < KB; ++kb, ++g, ld.next(p)) {
+        const int s = g % STAGES;
+        if (!mbar_wait(&empty[s], ((g / STAGES) & 1) ^ 1)) {
+          atomicExch(p.err, 4);
+          *abort_flag = 1;
+          break;
+        }
+        if (elect_one()) {
           char* sa = smem + s * STAGE_BYTES;
           mbar_expect_tx(&full[s], STAGE_BYTES);
-          load_kblock<KIND, BN, EPI>(p, kb, m0, n0, sa, sa + A_BYTES, &full[s]);
+          ld.load(p, sa, sa + A_BYTES, &full[s]);
         }
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = instr_desc(BN, KindTraits<KIND>::a_mn, KindTraits<KIND>::b_mn);
-      uint32_t g = 0, lt = 0;
-      for (int t = unit; t < tiles && !*abort_flag; t += units, ++lt) {
-        const uint32_t b = lt & 1;
-        // E_TMA: the epilogue warps arrive once per buffer before the first
-        // tile, after writing its starting value
-        if (!mbar_wait(&acc_empty[b], ((lt >> 1) & 1) ^ ((EPI & E_TMA) ? 0u : 1u))) {
-          atomicExch(p.err, 5);
+    uint32_t g = 0, lt = 0;
+    for (int t = unit; t < tiles && !*abort_flag; t += units, ++lt) {
+      const uint32_t b = lt & 1;
+      // E_TMA: the epilogue warps arrive once per buffer before the first
+      // tile, after writing its starting value
+      if (!mbar_wait(&acc_empty[b], ((lt >> 1) & 1) ^ ((EPI & E_TMA) ? 0u : 1u))) {
+        atomicExch(p.err, 5);
+        *abort_flag = 1;
+        if (elect_one()) mbar_expect_tx(&acc_full[b], 0);
+        break;
+      }
+      tc_fence_after();
+      const uint32_t d = tmem + b * BN;
+      bool ok = true;
+      for (int kb = 0; kb < KB; ++kb, ++g) {
+        const int s = g % STAGES;
+        if (!mbar_wait(&full[s], (g / STAGES) & 1)) {
+          atomicExch(p.err, 6);
           *abort_flag = 1;
-          mbar_expect_tx(&acc_full[b], 0);
+          ok = false;
           break;
         }
         tc_fence_after();
-        const uint32_t d = tmem + b * BN;
-        bool ok = true;
-        for (int kb = 0; kb < KB; ++kb, ++g) {
-          const int s = g % STAGES;
-          if (!mbar_wait(&full[s], (g / STAGES) & 1)) {
-            atomicExch(p.err, 6);
-            *abort_flag = 1;
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t a0 = smem_u32(smem + s * STAGE_BYTES);
-          const uint32_t b0 = a0 + A_BYTES;
-#pragma unroll
-          for (int k = 0; k < BK / UK; ++k) {
-            uint64_t ad, bd;
-            if (KindTraits<KIND>::a_mn) ad = smem_desc(a0 + k * UK * 128, BK * 128, 1024);
-            else ad = smem_desc(a0 + k * UK * 2, 16, 1024);
-            if (KindTraits<KIND>::b_mn) bd = smem_desc(b0 + k * UK * 128, BK * 128, 1024);
-            else bd = smem_desc(b0 + k * UK * 2, 16, 1024);
-            mma_f16(d, ad, bd, idesc, ((EPI & E_TMA) || kb > 0 || k > 0) ? 1u : 0u);
-          }
-          mma_commit(&empty[s]);
-        }
-        if (ok) mma_commit(&acc_full[b]);
-        else {
-          mbar_expect_tx(&acc_full[b], 0);
-          break;
-        }
+        if (elect_one())
+          mma_stage<KIND, BN>(d, smem_u32(smem + s * STAGE_BYTES), (EPI & E_TMA) || kb > 0, &empty[s]);
       }
+      if (elect_one()) {
+        if (ok) mma_commit(&acc_full[b]);
+        else mbar_expect_tx(&acc_full[b], 0);
+      }
+      if (!ok) break;
     }
   } else if constexpr ((EPI & E_TMA) != 0) {
     // Epilogue through TMA stores: warp w (2..9) owns TMEM lanes
