@@ -81,7 +81,7 @@ int* tc_error_word(TcContext* c);
 bool tc_encode_2d(CUtensorMap* m, const void* base, int64_t rows, int64_t cols, int box_rows);
 
 // Tensor-core attention (k_attention_tc.cu): sequences of at most 128 tokens,
-// head width 64, bf16.  A plan holds the tensor maps of the packed q|k|v
+// head widths 16, 32, 48 and 64, bf16.  A plan holds the tensor maps of the packed q|k|v
 // input [B*L, 3C] and of dO [B*L, C], and the address of the output O
 // [B*L, C] (the backward reads its rows directly).
 struct AttnTcPlan;

@@ -1,6 +1,6 @@
 // Tensor-core multi-head attention for sequences of up to 128 tokens and
-// head width 64 (bf16 activations): one CTA per (sequence, head), the whole
-// 128 x 128 score tile in TMEM.  Same operation as the CUDA-core kernels
+// head widths 16, 32, 48 and 64 (bf16 activations): one CTA per (sequence,
+// head), the whole 128 x 128 score tile in TMEM.  Same operation as the CUDA-core kernels
 // (scaled dot-product attention with keys j >= length[b] masked out):
 //   forward   S = Q K^T (TMEM) -> row maximum M of S / sqrt(64) -> P~ =
 //             exp(S / 8 - M) (bf16, shared memory) and its row sum ->
@@ -9,6 +9,16 @@
 //   backward  S = Q K^T and dP = dO V^T (TMEM) -> P = exp(S / 8 - lse),
 //             dS = P (dP - rowsum(dO * O)) / 8 (bf16, shared memory) ->
 //             dV = P^T dO, dQ = dS K, dK = dS^T Q (TMEM) -> d(q|k|v).
+// (8 stands for the square root of the head width DH.)  Tiles are always 64
+// columns wide: a narrower head's tile goes on into its neighbour's columns
+// (or zeros past the last), which the products over DH never read and whose
+// output columns are not stored.
+// Narrower heads multiply P and dS as the sum of two bf16 tiles (value and
+// remainder, 16 bits of mantissa; SPLIT), since those widths ran in fp32 on
+// the CUDA cores before; their products then cost twice the MMAs of a path
+// that waits on latency, not on the tensor pipe.  One 256-wide encoder block of
+// 19 x 77 tokens, 8 heads of 32: the CUDA-core kernels took 36.7 us forward and
+// 61.4 backward alone; the whole step went from 279 to 143 us.
 // Operand tiles are 128 rows x 64 bf16 (128-byte rows, 128-byte swizzle),
 // loaded by TMA from the packed q|k|v [B*L, 3C] and dO [B*L, C] (the
 // backward reads O's rows directly for rowsum(dO * O));
@@ -33,7 +43,6 @@ namespace {
 constexpr int kAttnThreads = 320;
 constexpr int kSoftmaxThreads = 256;      // warps 2..9
 constexpr int kTile = 16384;              // 128 rows x 64 bf16
-constexpr float kScale = 0.125f;          // 1 / sqrt(64)
 
 struct AttnParams {
   CUtensorMap tm_qkv;     // [B*L, 3C], box 64 x 128
@@ -57,16 +66,45 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
+// v[0..8) as bf16 into a tile's 16-byte unit at `hi` and, when SPLIT, the
+// remainders of that rounding at `lo`.
+template <bool SPLIT>
+__device__ __forceinline__ void st_unit(uint32_t hi, uint32_t lo, const float (&v)[8]) {
+  uint32_t h[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) h[q] = pack_bf16x2(v[2 * q], v[2 * q + 1]);
+  st_shared4(hi, h[0], h[1], h[2], h[3]);
+  if constexpr (SPLIT) {
+    uint32_t l[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const __nv_bfloat162 b = *reinterpret_cast<const __nv_bfloat162*>(&h[q]);
+      l[q] = pack_bf16x2(v[2 * q] - __low2float(b), v[2 * q + 1] - __high2float(b));
+    }
+    st_shared4(lo, l[0], l[1], l[2], l[3]);
+  }
+}
+
+template <bool SPLIT>
+__device__ __forceinline__ float attn_exp(float x) {
+  return SPLIT ? expf(x) : __expf(x);   // the widths that ran in fp32 keep the accurate one
+}
+template <int DH>
+__device__ __forceinline__ float attn_scale() {
+  return DH == 64 ? 0.125f : rsqrtf(float(DH));
+}
+
 __device__ __forceinline__ char* align1024(char* p) {
   return reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(p) + 1023) & ~uintptr_t(1023));
 }
 
-// 32 accumulator columns of this lane's row -> 32 bf16 at dst (optionally
-// added to what is there).
-__device__ __forceinline__ void store_row32(bf16* dst, const uint32_t (&r)[32], bool acc) {
+// The first N accumulator columns of this lane's row -> N bf16 at dst
+// (optionally added to what is there).
+template <int N>
+__device__ __forceinline__ void store_row(bf16* dst, const uint32_t (&r)[32], bool acc) {
   uint4* d4 = reinterpret_cast<uint4*>(dst);
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
+  for (int q = 0; q < N / 8; ++q) {
     float v[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) v[e] = __uint_as_float(r[8 * q + e]);
@@ -81,13 +119,18 @@ __device__ __forceinline__ void store_row32(bf16* dst, const uint32_t (&r)[32], 
   }
 }
 
+template <int DH, bool SPLIT>
 __global__ void __launch_bounds__(kAttnThreads, 1) attn_fwd_tc_k(const __grid_constant__ AttnParams p) {
   extern __shared__ __align__(1024) char smem_raw[];
   char* sm = align1024(smem_raw);
   char* sQ = sm;
   char* sK = sm + kTile;
   char* sV = sm + 2 * kTile;
-  char* sP = sm + 3 * kTile;                       // two sub-tiles (keys 0..63, 64..127)
+  // P~: two sub-tiles (keys 0..63, 64..127); SPLIT: the values over Q and K,
+  // which S = Q K^T alone reads, and the remainders in the two tiles after V
+  char* sP = SPLIT ? sm : sm + 3 * kTile;
+  char* sPlo = sm + 3 * kTile;
+  const float kScale = attn_scale<DH>();
   uint64_t* bars = reinterpret_cast<uint64_t*>(sm + 5 * kTile);   // ld, s, p, o
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 4);
   float2* xch = reinterpret_cast<float2*>(sm + 5 * kTile + 64);   // [half][row]: partial maxima, then sums
@@ -119,9 +162,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_fwd_tc_k(const __grid_co
   if (warp == 0) {
     if (lane == 0) {
       mbar_expect_tx(&bars[0], 3 * kTile);
-      tma_2d(sQ, &p.tm_qkv, &bars[0], h * 64, row0);
-      tma_2d(sK, &p.tm_qkv, &bars[0], p.C + h * 64, row0);
-      tma_2d(sV, &p.tm_qkv, &bars[0], 2 * p.C + h * 64, row0);
+      tma_2d(sQ, &p.tm_qkv, &bars[0], h * DH, row0);
+      tma_2d(sK, &p.tm_qkv, &bars[0], p.C + h * DH, row0);
+      tma_2d(sV, &p.tm_qkv, &bars[0], 2 * p.C + h * DH, row0);
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -129,7 +172,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_fwd_tc_k(const __grid_co
       tc_fence_after();
       constexpr uint32_t id_s = instr_desc(128, false, false);
 #pragma unroll
-      for (int k = 0; k < 4; ++k)
+      for (int k = 0; k < DH / 16; ++k)
         mma_f16(tmem, smem_desc(smem_u32(sQ) + 32 * k, 16, 1024), smem_desc(smem_u32(sK) + 32 * k, 16, 1024), id_s,
                 k > 0 ? 1u : 0u);
       mma_commit(&bars[1]);
@@ -140,6 +183,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_fwd_tc_k(const __grid_co
       for (int k = 0; k < 8; ++k)
         mma_f16(tmem + 128, smem_desc(smem_u32(sP) + (k >> 2) * kTile + 32 * (k & 3), 16, 1024),
                 smem_desc(smem_u32(sV) + 2048 * k, kTile, 1024), id_o, k > 0 ? 1u : 0u);
+      if constexpr (SPLIT)
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          mma_f16(tmem + 128, smem_desc(smem_u32(sPlo) + (k >> 2) * kTile + 32 * (k & 3), 16, 1024),
+                  smem_desc(smem_u32(sV) + 2048 * k, kTile, 1024), id_o, 1u);
       mma_commit(&bars[3]);
     }
   } else {
@@ -166,6 +214,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_fwd_tc_k(const __grid_co
     // its row sum; O = P~ V is normalised by the sum in the store below
     float sum = 0.f;
     const uint32_t p_base = smem_u32(sP) + uint32_t(hf) * kTile;
+    const uint32_t l_base = smem_u32(sPlo) + uint32_t(hf) * kTile;
 #pragma unroll 1
     for (int c = 0; c < 2; ++c) {
       tmem_ld32(trow + 32 * c, r);
@@ -175,11 +224,10 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_fwd_tc_k(const __grid_co
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           const int j = 64 * hf + 32 * c + 8 * g + e;
-          v[e] = j < n ? __expf(__uint_as_float(r[8 * g + e]) * kScale - M) : 0.f;
+          v[e] = j < n ? attn_exp<SPLIT>(__uint_as_float(r[8 * g + e]) * kScale - M) : 0.f;
           sum += v[e];
         }
-        st_shared4(p_base + sw_off(i, c * 4 + g), pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]),
-                   pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
+        st_unit<SPLIT>(p_base + sw_off(i, c * 4 + g), l_base + sw_off(i, c * 4 + g), v);
       }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // P~ visible to the tensor cores
@@ -193,11 +241,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_fwd_tc_k(const __grid_co
     if (hf == 0 && i < p.L) p.lse[size_t(bh) * p.L + i] = M + logf(S);
     if (!mbar_wait(&bars[3], 0)) atomicExch(p.err, 14);
     tc_fence_after();
-    // O: 64 columns at TMEM column 128; each half of the pair stores 32
-    tmem_ld32(tmem + (uint32_t(q * 32) << 16) + 128 + 32 * hf, r);
+    // O: DH columns from TMEM column 128 on; each half of the pair stores half of them
+    tmem_ld32(tmem + (uint32_t(q * 32) << 16) + 128 + DH / 2 * hf, r);
 #pragma unroll
     for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) * inv);
-    if (i < p.L) store_row32(p.out + size_t(row0 + i) * p.C + h * 64 + 32 * hf, r, false);
+    if (i < p.L) store_row<DH / 2>(p.out + size_t(row0 + i) * p.C + h * DH + DH / 2 * hf, r, false);
   }
   tc_fence_before();
   __syncthreads();
@@ -212,7 +260,9 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_fwd_tc_k(const __grid_co
 // buffer once that phase has completed; O is read from global memory (only
 // its row sums with dO are needed); dQ, dV and dK take the TMEM columns of S
 // and dP, which the softmax warps have read before the second phase starts.
-__global__ void __launch_bounds__(kAttnThreads, 2) attn_bwd_tc_k(const __grid_constant__ AttnParams p) {
+// SPLIT: four more tiles hold the remainders of P and dS, one CTA per SM.
+template <int DH, bool SPLIT>
+__global__ void __launch_bounds__(kAttnThreads, SPLIT ? 1 : 2) attn_bwd_tc_k(const __grid_constant__ AttnParams p) {
   extern __shared__ __align__(1024) char smem_raw[];
   char* sm = align1024(smem_raw);
   char* sQ = sm;
@@ -221,10 +271,13 @@ __global__ void __launch_bounds__(kAttnThreads, 2) attn_bwd_tc_k(const __grid_co
   char* sP = sm + 2 * kTile;      // two sub-tiles: V's buffer after the first phase, then the next
   char* sdO = sm + 4 * kTile;
   char* sdS = sm + 5 * kTile;     // two sub-tiles
+  char* sPlo = sm + 7 * kTile;    // SPLIT: two sub-tiles each
+  char* sdSlo = sm + 9 * kTile;
+  const float kScale = attn_scale<DH>();
   // barriers (ld, s, p, g) and the TMEM slot: in the alignment slack below
   // the tiles when it has room, else after them (the request covers both)
   const bool low = sm - smem_raw >= 64;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(low ? smem_raw : sm + 7 * kTile);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(low ? smem_raw : sm + (SPLIT ? 11 : 7) * kTile);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 4);
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -256,10 +309,10 @@ __global__ void __launch_bounds__(kAttnThreads, 2) attn_bwd_tc_k(const __grid_co
   if (warp == 0) {
     if (lane == 0) {
       mbar_expect_tx(&bars[0], 4 * kTile);
-      tma_2d(sQ, &p.tm_qkv, &bars[0], h * 64, row0);
-      tma_2d(sK, &p.tm_qkv, &bars[0], p.C + h * 64, row0);
-      tma_2d(sV, &p.tm_qkv, &bars[0], 2 * p.C + h * 64, row0);
-      tma_2d(sdO, &p.tm_do, &bars[0], h * 64, row0);
+      tma_2d(sQ, &p.tm_qkv, &bars[0], h * DH, row0);
+      tma_2d(sK, &p.tm_qkv, &bars[0], p.C + h * DH, row0);
+      tma_2d(sV, &p.tm_qkv, &bars[0], 2 * p.C + h * DH, row0);
+      tma_2d(sdO, &p.tm_do, &bars[0], h * DH, row0);
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -267,7 +320,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) attn_bwd_tc_k(const __grid_co
       tc_fence_after();
       constexpr uint32_t id_nn128 = instr_desc(128, false, false);
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
+      for (int k = 0; k < DH / 16; ++k) {
         mma_f16(tmem, smem_desc(smem_u32(sQ) + 32 * k, 16, 1024), smem_desc(smem_u32(sK) + 32 * k, 16, 1024),
                 id_nn128, k > 0 ? 1u : 0u);
         mma_f16(tmem + 128, smem_desc(smem_u32(sdO) + 32 * k, 16, 1024),
@@ -291,6 +344,16 @@ __global__ void __launch_bounds__(kAttnThreads, 2) attn_bwd_tc_k(const __grid_co
         mma_f16(tmem + 192, smem_desc(smem_u32(sdS) + 2048 * k, kTile, 1024),
                 smem_desc(smem_u32(sQ) + 2048 * k, kTile, 1024), id_tt, acc);
       }
+      if constexpr (SPLIT)
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {   // the same products of the remainders
+          mma_f16(tmem + 128, smem_desc(smem_u32(sPlo) + 2048 * k, kTile, 1024),
+                  smem_desc(smem_u32(sdO) + 2048 * k, kTile, 1024), id_tt, 1u);
+          mma_f16(tmem, smem_desc(smem_u32(sdSlo) + (k >> 2) * kTile + 32 * (k & 3), 16, 1024),
+                  smem_desc(smem_u32(sK) + 2048 * k, kTile, 1024), id_nt, 1u);
+          mma_f16(tmem + 192, smem_desc(smem_u32(sdSlo) + 2048 * k, kTile, 1024),
+                  smem_desc(smem_u32(sQ) + 2048 * k, kTile, 1024), id_tt, 1u);
+        }
       mma_commit(&bars[3]);
     }
   } else {
@@ -300,19 +363,19 @@ __global__ void __launch_bounds__(kAttnThreads, 2) attn_bwd_tc_k(const __grid_co
     const bool live = i < p.L;          // rows past the sequence get P = dS = 0
     // D_i = sum_d dO[i][d] O[i][d]: O's row from global memory (in flight
     // during the TMA wait), dO's from the swizzled tile
-    uint4 orow[8];
+    uint4 orow[DH / 8];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) orow[u] = make_uint4(0u, 0u, 0u, 0u);
+    for (int u = 0; u < DH / 8; ++u) orow[u] = make_uint4(0u, 0u, 0u, 0u);
     if (live) {
-      const uint4* src = reinterpret_cast<const uint4*>(p.o + size_t(row0 + i) * p.C + h * 64);
+      const uint4* src = reinterpret_cast<const uint4*>(p.o + size_t(row0 + i) * p.C + h * DH);
 #pragma unroll
-      for (int u = 0; u < 8; ++u) orow[u] = src[u];
+      for (int u = 0; u < DH / 8; ++u) orow[u] = src[u];
     }
     if (!mbar_wait(&bars[0], 0)) atomicExch(p.err, 15);
     float D = 0.f;
     const uint32_t do_base = smem_u32(sdO);
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
+    for (int u = 0; u < DH / 8; ++u) {
       const float4 a = ld_shared4(do_base + sw_off(i, u));
       const bf16* ab = reinterpret_cast<const bf16*>(&a);
       const bf16* cb = reinterpret_cast<const bf16*>(&orow[u]);
@@ -323,6 +386,7 @@ __global__ void __launch_bounds__(kAttnThreads, 2) attn_bwd_tc_k(const __grid_co
     if (!mbar_wait(&bars[1], 0)) atomicExch(p.err, 13);
     tc_fence_after();
     const uint32_t p_base = smem_u32(sP), ds_base = smem_u32(sdS);
+    const uint32_t pl_base = smem_u32(sPlo), dsl_base = smem_u32(sdSlo);
 #pragma unroll 1
     for (int c = 2 * hf; c < 2 * hf + 2; ++c) {
       uint32_t rs[32], rp[32];
@@ -334,15 +398,13 @@ __global__ void __launch_bounds__(kAttnThreads, 2) attn_bwd_tc_k(const __grid_co
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           const int j = 32 * c + 8 * g + e;
-          const float pj = (live && j < n) ? __expf(__uint_as_float(rs[8 * g + e]) * kScale - lse) : 0.f;
+          const float pj = (live && j < n) ? attn_exp<SPLIT>(__uint_as_float(rs[8 * g + e]) * kScale - lse) : 0.f;
           pv[e] = pj;
           dv[e] = pj * (__uint_as_float(rp[8 * g + e]) - D) * kScale;
         }
         const uint32_t off = (c >> 1) * kTile + sw_off(i, (c & 1) * 4 + g);
-        st_shared4(p_base + off, pack_bf16x2(pv[0], pv[1]), pack_bf16x2(pv[2], pv[3]), pack_bf16x2(pv[4], pv[5]),
-                   pack_bf16x2(pv[6], pv[7]));
-        st_shared4(ds_base + off, pack_bf16x2(dv[0], dv[1]), pack_bf16x2(dv[2], dv[3]), pack_bf16x2(dv[4], dv[5]),
-                   pack_bf16x2(dv[6], dv[7]));
+        st_unit<SPLIT>(p_base + off, pl_base + off, pv);
+        st_unit<SPLIT>(ds_base + off, dsl_base + off, dv);
       }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // P, dS visible to the tensor cores
@@ -351,14 +413,14 @@ __global__ void __launch_bounds__(kAttnThreads, 2) attn_bwd_tc_k(const __grid_co
     if (!mbar_wait(&bars[3], 0)) atomicExch(p.err, 14);
     tc_fence_after();
     // TMEM row i holds dQ row i and dK / dV row j = i; each half of the
-    // pair stores 32 of the 64 columns of each
+    // pair stores half of the DH columns of each
     bf16* drow = p.out + size_t(row0 + i) * 3 * p.C;
 #pragma unroll 1
     for (int t = 0; t < 3; ++t) {
       const uint32_t col = t == 0 ? 0u : (t == 1 ? 192u : 128u);     // dQ, dK, dV
       uint32_t r[32];
-      tmem_ld32(trow + col + 32 * hf, r);
-      if (live) store_row32(drow + t * p.C + h * 64 + 32 * hf, r, p.acc != 0);
+      tmem_ld32(trow + col + DH / 2 * hf, r);
+      if (live) store_row<DH / 2>(drow + t * p.C + h * DH + DH / 2 * hf, r, p.acc != 0);
     }
   }
   tc_fence_before();
@@ -371,20 +433,43 @@ __global__ void __launch_bounds__(kAttnThreads, 2) attn_bwd_tc_k(const __grid_co
 
 constexpr size_t kFwdSmem = 5 * kTile + 1024 + 64 + 4 * 128 * sizeof(float2);
 constexpr size_t kBwdSmem = 7 * kTile + 1024;   // 115,712 B: two CTAs in an SM's 228 KB
+constexpr size_t kBwdSplitSmem = 11 * kTile + 1024;
+
+typedef void (*AttnKernel)(const AttnParams);
+struct AttnKernels {
+  AttnKernel fwd, bwd;
+  size_t bwd_smem;
+};
+// The kernels of a head width, or nulls.
+AttnKernels attn_kernels(int dh) {
+  switch (dh) {
+    case 16: return {attn_fwd_tc_k<16, true>, attn_bwd_tc_k<16, true>, kBwdSplitSmem};
+    case 32: return {attn_fwd_tc_k<32, true>, attn_bwd_tc_k<32, true>, kBwdSplitSmem};
+    case 48: return {attn_fwd_tc_k<48, true>, attn_bwd_tc_k<48, true>, kBwdSplitSmem};
+    case 64: return {attn_fwd_tc_k<64, false>, attn_bwd_tc_k<64, false>, kBwdSmem};
+  }
+  return {nullptr, nullptr, 0};
+}
 
 }  // namespace
 
 struct AttnTcPlan {
   AttnParams p;
+  AttnKernels k;
 };
 
-bool attention_tc_ok(int L, int C, int heads) { return L >= 1 && L <= 128 && heads > 0 && C == 64 * heads; }
+// Head widths that are multiples of the MMA's K of 16 (so every box also
+// starts on a 16-byte boundary); others stay on the CUDA cores.
+bool attention_tc_ok(int L, int C, int heads) {
+  return L >= 1 && L <= 128 && heads > 0 && C % heads == 0 && attn_kernels(C / heads).fwd != nullptr;
+}
 
 AttnTcPlan* attention_tc_plan(const void* qkv, const void* out, const void* dout, int B, int L, int C, int heads,
                               int* err) {
   if (!attention_tc_ok(L, C, heads)) return nullptr;
   AttnTcPlan* a = new AttnTcPlan();
   a->p = AttnParams{};
+  a->k = attn_kernels(C / heads);
   a->p.L = L;
   a->p.C = C;
   a->p.heads = heads;
@@ -396,16 +481,14 @@ AttnTcPlan* attention_tc_plan(const void* qkv, const void* out, const void* dout
     delete a;
     return nullptr;
   }
-  // Both kernels are sized for two CTAs per SM, which needs the largest
-  // shared-memory carveout (the default sizes the carveout for one block).
-  if (cudaFuncSetAttribute(attn_fwd_tc_k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kFwdSmem)) !=
-          cudaSuccess ||
-      cudaFuncSetAttribute(attn_bwd_tc_k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kBwdSmem)) !=
-          cudaSuccess ||
-      cudaFuncSetAttribute(attn_fwd_tc_k, cudaFuncAttributePreferredSharedMemoryCarveout,
-                           int(cudaSharedmemCarveoutMaxShared)) != cudaSuccess ||
-      cudaFuncSetAttribute(attn_bwd_tc_k, cudaFuncAttributePreferredSharedMemoryCarveout,
-                           int(cudaSharedmemCarveoutMaxShared)) != cudaSuccess) {
+  // Sized for two CTAs per SM (the backward of the narrower heads for one),
+  // which needs the largest shared-memory carveout (the default sizes the
+  // carveout for one block).
+  const int most = int(cudaSharedmemCarveoutMaxShared);
+  if (cudaFuncSetAttribute(a->k.fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kFwdSmem)) != cudaSuccess ||
+      cudaFuncSetAttribute(a->k.bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, int(a->k.bwd_smem)) != cudaSuccess ||
+      cudaFuncSetAttribute(a->k.fwd, cudaFuncAttributePreferredSharedMemoryCarveout, most) != cudaSuccess ||
+      cudaFuncSetAttribute(a->k.bwd, cudaFuncAttributePreferredSharedMemoryCarveout, most) != cudaSuccess) {
     delete a;
     return nullptr;
   }
@@ -420,7 +503,7 @@ void attention_tc_fwd(const AttnTcPlan* a, const int32_t* len, void* out, float*
   p.out = static_cast<bf16*>(out);
   p.lse = lse;
   p.acc = 0;
-  launch_k(attn_fwd_tc_k, B * p.heads, kAttnThreads, kFwdSmem, st, p);
+  launch_k(a->k.fwd, B * p.heads, kAttnThreads, kFwdSmem, st, p);
 }
 
 void attention_tc_bwd(const AttnTcPlan* a, const int32_t* len, const float* lse, void* dqkv, int B, bool acc,
@@ -430,7 +513,7 @@ void attention_tc_bwd(const AttnTcPlan* a, const int32_t* len, const float* lse,
   p.out = static_cast<bf16*>(dqkv);
   p.lse = const_cast<float*>(lse);
   p.acc = acc ? 1 : 0;
-  launch_k(attn_bwd_tc_k, B * p.heads, kAttnThreads, kBwdSmem, st, p);
+  launch_k(a->k.bwd, B * p.heads, kAttnThreads, a->k.bwd_smem, st, p);
 }
 
 }  // namespace fo
