@@ -173,23 +173,23 @@ void affine_bwd8_pass(const void* dy, const void* x, const float* scale, void* d
 // Affine then hard swish in one pass: pre = x * scale + shift, post = hswish(pre).
 void affine_hswish_fwd_x8(const void* x, const float* sc, const float* sh, void* pre, void* post, int64_t n, int C,
                           cudaStream_t st);
-// Layernorm forward with the row in registers (bf16, C % 256 == 0, C <= 1024).
+// Layernorm forward with the row in registers (bf16, C % 8 == 0, C <= 1024).
 bool layernorm_fwd8_ok(int dt, int C);
 void layernorm_fwd_x8(const void* x, const float* gamma, const float* beta, void* y, float* mean, float* rstd,
                       int64_t rows, int C, cudaStream_t st);
-// Layernorm backward fused with dgamma / dbeta (C % 256 == 0, C <= 512).
+// Layernorm backward fused with dgamma / dbeta (bf16, C % 8 == 0, C <= 1024).
 // Masked mean-pool over tokens and its gradient, 8 bf16 columns per access.
 bool meanpool8_ok(int dt, int C);
 void meanpool_fwd_x8(const void* x, const int32_t* len, void* y, int B, int L, int C, cudaStream_t st);
 void meanpool_bwd_x8(const void* dy, const int32_t* len, void* dx, int B, int L, int C, bool acc, cudaStream_t st);
 bool layernorm_bwd8_ok(int dt, int C);
 int64_t layernorm_bwd8_partial_floats(int64_t rows, int C);
-// The same pass without its finish: partials [layernorm_bwd8_blocks(rows), C]
+// The same pass without its finish: partials [layernorm_bwd8_blocks(rows, C), C]
 // of dgamma and dbeta.
-int layernorm_bwd8_blocks(int64_t rows);
+int layernorm_bwd8_blocks(int64_t rows, int C);
 // dx = (dx if acc) + input gradient + (addend if given, dx's layout).
 // With p_dx, also the column partial sums of the stored dx per block
-// ([layernorm_bwd8_blocks(rows)][C]): the bias gradient of the layer whose
+// ([layernorm_bwd8_blocks(rows, C)][C]): the bias gradient of the layer whose
 // output gradient dx is.
 void layernorm_bwd8_pass(const void* x, const float* gamma, const float* mean, const float* rstd, const void* dy,
                          void* dx, int64_t rows, int C, bool acc, float* p_gamma, float* p_beta, cudaStream_t st,

@@ -900,10 +900,10 @@ int build_plan(fo_server* s) {
           const void* addend = nullptr;
           const int accf = need_dx ? contrib_addend(a, &addend) : 0;
           auto req = std::make_shared<PartReq>();
-          req->chunks = fo::layernorm_bwd8_blocks(s->T[a0].rows());
+          req->chunks = fo::layernorm_bwd8_blocks(s->T[a0].rows(), s->T[a0].C);
           if (need_dx) last_part[groot(a)] = req;
           const Tensor& x0 = s->T[a0];
-          const int blocks = fo::layernorm_bwd8_blocks(x0.rows());
+          const int blocks = fo::layernorm_bwd8_blocks(x0.rows(), x0.C);
           float* pg = (float*)s->alloc(size_t(2) * blocks * x0.C * 4);
           if (!pg) return set_err(FO_ERR_OOM, "layernorm partials");
           float* pb = pg + size_t(blocks) * x0.C;

@@ -309,8 +309,9 @@ __global__ void __launch_bounds__(256) colsum8_batch_k(const __grid_constant__ C
                    local % cbs, local / cbs);
 }
 
-// Layernorm forward, rows held in registers (C = 256 NV, NV <= 4, a
-// template parameter so that a row takes only the registers it needs): each
+// Layernorm forward, rows held in registers (C <= 256 NV, C % 8 == 0, NV <= 4,
+// a template parameter so that a row takes only the registers it needs; lanes
+// whose vector lies past C hold zeros and stay out of the variance): each
 // warp takes R consecutive rows and loads all of them before any
 // arithmetic; one read of x, mean then biased variance from the registers
 // (eps 1e-5), one write of y; the row mean and 1/std are kept for the
@@ -333,11 +334,12 @@ __global__ void __launch_bounds__(256, 2) layernorm_fwd_x8_k(const bf16* __restr
   for (int r = 0; r < R; ++r)
 #pragma unroll
     for (int v = 0; v < NV; ++v)
-      xr[r][v] = row0 + r < rows ? *reinterpret_cast<const uint4*>(x + (row0 + r) * C + (v * 32 + lane) * 8)
-                                 : make_uint4(0u, 0u, 0u, 0u);
+      xr[r][v] = row0 + r < rows && (v * 32 + lane) * 8 < C
+                     ? *reinterpret_cast<const uint4*>(x + (row0 + r) * C + (v * 32 + lane) * 8)
+                     : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
-    const int c = (v * 32 + lane) * 8;
+    const int c = (v * 32 + lane) * 8 < C ? (v * 32 + lane) * 8 : 0;
     g4[v][0] = __ldg(reinterpret_cast<const float4*>(gamma + c));
     g4[v][1] = __ldg(reinterpret_cast<const float4*>(gamma + c) + 1);
     b4[v][0] = __ldg(reinterpret_cast<const float4*>(beta + c));
@@ -361,7 +363,7 @@ __global__ void __launch_bounds__(256, 2) layernorm_fwd_x8_k(const bf16* __restr
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
         const float d = __bfloat162float(reinterpret_cast<const bf16*>(&xr[r][v])[j]) - mu;
-        q = fmaf(d, d, q);
+        if ((v * 32 + lane) * 8 < C) q = fmaf(d, d, q);
       }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
@@ -375,7 +377,7 @@ __global__ void __launch_bounds__(256, 2) layernorm_fwd_x8_k(const bf16* __restr
 #pragma unroll
       for (int j = 0; j < 8; ++j)
         o.v[j] = (__bfloat162float(reinterpret_cast<const bf16*>(&xr[r][v])[j]) - mu) * rs * gm[j] + bt[j];
-      st8(y + row * C + c, o);
+      if (c < C) st8(y + row * C + c, o);
     }
     if (lane == 0) {
       mean_out[row] = mu;
@@ -385,18 +387,23 @@ __global__ void __launch_bounds__(256, 2) layernorm_fwd_x8_k(const bf16* __restr
 }
 
 // Layernorm backward fused with its parameter gradients.  Each warp takes
-// kLnRows consecutive rows (a block kLnWarps kLnRows), with all of their operands
+// ln_rows(C) consecutive rows (a block kLnWarps times that), with all of their operands
 // loaded before any arithmetic.  The column partials of dy * xhat (gamma),
 // dy (beta) and, with pdx, of the stored dx accumulate in registers over the
 // warp's rows and are added over the block's warps, in warp order, through
 // shared memory once per block: exchanged row by row, those partials cost
-// more than the rest of the pass.  C <= 512, C % 256 == 0; dx may be null (a
+// more than the rest of the pass.  C <= 256 NV, C % 8 == 0 (lanes whose vector
+// lies past C hold zeros); dx may be null (a
 // layernorm of the uploaded batch has no input gradient).  dx receives the
 // layernorm's input gradient plus the NX extra operands ex0, ex1 (same
 // layout): its own old value when accumulating, and the gradient a residual
 // connection passes around the layernorm.
-constexpr int kLnRows = 4;
+// Widths that are no multiple of 256, and 768 and 1024, ran as a scalar pass
+// and four column-sum launches before: a step of one encoder block at batch 16
+// x 100 tokens, us: 384 wide 222 -> 171, 768 wide 295 -> 239 (with the
+// classifier head's change).
 constexpr int kLnWarps = 4;   // warps per block: the 4096-row step in 256 blocks
+constexpr int ln_rows_nv(int nv) { return nv <= 2 ? 4 : 2; }   // rows per warp: what its registers hold
 __device__ __forceinline__ float bf_at(const uint4& u, int j) {
   return __bfloat162float(reinterpret_cast<const bf16*>(&u)[j]);
 }
@@ -408,7 +415,7 @@ __global__ void __launch_bounds__(kLnWarps * 32, 1) layernorm_bwd_fused_k(const 
                                                                 float* __restrict__ pb, float* __restrict__ pdx) {
   pdl_wait();
   pdl_trigger();
-  constexpr int kMaxV = NV, nv = NV, CC = 256 * NV;   // 8-wide vectors per lane: C = 256 NV
+  constexpr int kMaxV = NV, nv = NV, kLnRows = ln_rows_nv(NV);   // 8-wide vectors per lane
   __shared__ __align__(16) float red[3][kLnWarps][256 * NV];
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int64_t row0 = (int64_t(blockIdx.x) * kLnWarps + warp) * kLnRows;
@@ -416,7 +423,7 @@ __global__ void __launch_bounds__(kLnWarps * 32, 1) layernorm_bwd_fused_k(const 
   float gm[kMaxV][8];
 #pragma unroll
   for (int v = 0; v < kMaxV; ++v) {
-    const int c = v < nv ? (v * 32 + lane) * 8 : 0;
+    const int c = (v * 32 + lane) * 8 < C ? (v * 32 + lane) * 8 : 0;
     const float4 g0 = __ldg(reinterpret_cast<const float4*>(gamma + c));
     const float4 g1 = __ldg(reinterpret_cast<const float4*>(gamma + c) + 1);
     gm[v][0] = g0.x; gm[v][1] = g0.y; gm[v][2] = g0.z; gm[v][3] = g0.w;
@@ -430,8 +437,8 @@ __global__ void __launch_bounds__(kLnWarps * 32, 1) layernorm_bwd_fused_k(const 
     const bool live = row < rows;
 #pragma unroll
     for (int v = 0; v < kMaxV; ++v) {
-      const bool ok = live && v < nv;
-      const int64_t off = row * CC + (v * 32 + lane) * 8;
+      const bool ok = live && (v * 32 + lane) * 8 < C;
+      const int64_t off = row * C + (v * 32 + lane) * 8;
       xr[r][v] = ok ? *reinterpret_cast<const uint4*>(x + off) : z;
       gr[r][v] = ok ? *reinterpret_cast<const uint4*>(dy + off) : z;
       if constexpr (NX > 0) er[r][v][0] = ok ? *reinterpret_cast<const uint4*>(ex0 + off) : z;
@@ -463,8 +470,8 @@ __global__ void __launch_bounds__(kLnWarps * 32, 1) layernorm_bwd_fused_k(const 
       a += __shfl_xor_sync(0xffffffffu, a, o);
       b += __shfl_xor_sync(0xffffffffu, b, o);
     }
-    a *= 1.f / float(CC);
-    b *= 1.f / float(CC);
+    a *= 1.f / float(C);
+    b *= 1.f / float(C);
     if constexpr (DXP > 0) {
 #pragma unroll
       for (int v = 0; v < kMaxV; ++v) {
@@ -478,9 +485,9 @@ __global__ void __launch_bounds__(kLnWarps * 32, 1) layernorm_bwd_fused_k(const 
           if constexpr (NX > 0) val += bf_at(er[r][v][0], j);
           if constexpr (NX > 1) val += bf_at(er[r][v][1], j);
           ob[j] = __float2bfloat16_rn(val);
-          if constexpr (DXP == 2) ax[v][j] += live ? __bfloat162float(ob[j]) : 0.f;   // the stored value
+          if constexpr (DXP == 2) ax[v][j] += live ? __bfloat162float(ob[j]) : 0.f;   // the stored value (columns past C unused)
         }
-        if (live) *reinterpret_cast<uint4*>(dx + row * CC + (v * 32 + lane) * 8) = o;
+        if (live && (v * 32 + lane) * 8 < C) *reinterpret_cast<uint4*>(dx + row * C + (v * 32 + lane) * 8) = o;
       }
     }
   }
@@ -766,11 +773,14 @@ void finish_batched(const std::vector<FinishTask>& tasks, cudaStream_t st) {
   }
 }
 
-bool layernorm_bwd8_ok(int dt, int C) { return dt == kBF16 && C % 256 == 0 && C <= 512; }
+bool layernorm_bwd8_ok(int dt, int C) { return dt == kBF16 && C % 8 == 0 && C <= 1024; }
 
-int layernorm_bwd8_blocks(int64_t rows) { return int((rows + kLnWarps * kLnRows - 1) / (kLnWarps * kLnRows)); }
+int layernorm_bwd8_blocks(int64_t rows, int C) {
+  const int per = kLnWarps * ln_rows_nv((C + 255) / 256);
+  return int((rows + per - 1) / per);
+}
 
-bool layernorm_fwd8_ok(int dt, int C) { return dt == kBF16 && C % 256 == 0 && C <= 1024; }
+bool layernorm_fwd8_ok(int dt, int C) { return dt == kBF16 && C % 8 == 0 && C <= 1024; }
 void layernorm_fwd_x8(const void* x, const float* gamma, const float* beta, void* y, float* mean, float* rstd,
                       int64_t rows, int C, cudaStream_t st) {
   if (C <= 512) {
@@ -790,20 +800,26 @@ void layernorm_bwd8_pass(const void* x, const float* gamma, const float* mean, c
   if (dx && acc) ex[nx++] = static_cast<const bf16*>(dx);
   if (dx && addend) ex[nx++] = static_cast<const bf16*>(addend);
   using K = decltype(&layernorm_bwd_fused_k<0, 1, 0>);
-  static const K table[2][3][3] = {   // [NV - 1][NX][DXP]; NX > 0 comes with a dx
+  static const K table[4][3][3] = {   // [NV - 1][NX][DXP]; NX > 0 comes with a dx
       {{layernorm_bwd_fused_k<0, 1, 0>, layernorm_bwd_fused_k<0, 1, 1>, layernorm_bwd_fused_k<0, 1, 2>},
        {nullptr, layernorm_bwd_fused_k<1, 1, 1>, layernorm_bwd_fused_k<1, 1, 2>},
        {nullptr, layernorm_bwd_fused_k<2, 1, 1>, layernorm_bwd_fused_k<2, 1, 2>}},
       {{layernorm_bwd_fused_k<0, 2, 0>, layernorm_bwd_fused_k<0, 2, 1>, layernorm_bwd_fused_k<0, 2, 2>},
        {nullptr, layernorm_bwd_fused_k<1, 2, 1>, layernorm_bwd_fused_k<1, 2, 2>},
-       {nullptr, layernorm_bwd_fused_k<2, 2, 1>, layernorm_bwd_fused_k<2, 2, 2>}}};
+       {nullptr, layernorm_bwd_fused_k<2, 2, 1>, layernorm_bwd_fused_k<2, 2, 2>}},
+      {{layernorm_bwd_fused_k<0, 3, 0>, layernorm_bwd_fused_k<0, 3, 1>, layernorm_bwd_fused_k<0, 3, 2>},
+       {nullptr, layernorm_bwd_fused_k<1, 3, 1>, layernorm_bwd_fused_k<1, 3, 2>},
+       {nullptr, layernorm_bwd_fused_k<2, 3, 1>, layernorm_bwd_fused_k<2, 3, 2>}},
+      {{layernorm_bwd_fused_k<0, 4, 0>, layernorm_bwd_fused_k<0, 4, 1>, layernorm_bwd_fused_k<0, 4, 2>},
+       {nullptr, layernorm_bwd_fused_k<1, 4, 1>, layernorm_bwd_fused_k<1, 4, 2>},
+       {nullptr, layernorm_bwd_fused_k<2, 4, 1>, layernorm_bwd_fused_k<2, 4, 2>}}};
   const int dxp = dx ? (p_dx ? 2 : 1) : 0;
-  auto k = table[C <= 256 ? 0 : 1][nx][dxp];
-  launch_k(k, layernorm_bwd8_blocks(rows), kLnWarps * 32, 0, st, (const bf16*)x, gamma, mean, rstd, (const bf16*)dy, (bf16*)dx,
+  auto k = table[(C + 255) / 256 - 1][nx][dxp];
+  launch_k(k, layernorm_bwd8_blocks(rows, C), kLnWarps * 32, 0, st, (const bf16*)x, gamma, mean, rstd, (const bf16*)dy, (bf16*)dx,
            rows, C, ex[0], ex[1], p_gamma, p_beta, dx ? p_dx : nullptr);
 }
 
-int64_t layernorm_bwd8_partial_floats(int64_t rows, int C) { return 2 * int64_t(layernorm_bwd8_blocks(rows)) * C; }
+int64_t layernorm_bwd8_partial_floats(int64_t rows, int C) { return 2 * int64_t(layernorm_bwd8_blocks(rows, C)) * C; }
 
 bool meanpool8_ok(int dt, int C) { return dt == kBF16 && C % 8 == 0; }
 void meanpool_fwd_x8(const void* x, const int32_t* len, void* y, int B, int L, int C, cudaStream_t st) {
