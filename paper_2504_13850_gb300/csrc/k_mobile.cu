@@ -201,6 +201,178 @@ __global__ void __launch_bounds__(256) dwconv_wgrad_any_k(const T* __restrict__ 
   }
 }
 
+// ------------------------------------------- depthwise conv, 8 channels wide
+// The bf16 kernels for k = 3, 5 and channel counts that are multiples of 8:
+// a thread owns 8 channels (one 16-byte access per tap), a block 64 channels,
+// whose weights it stages once as fp32 [tap][channel].  The scalar kernels
+// above read a channel's k * k weights with a stride of k * k elements and
+// divide 64-bit indices per element, which bounded them.  Steps, us, scalar ->
+// here: MobileNet part on 4 x 4 maps at batch 64 417 -> 394; on 14 x 14 maps at
+// batch 32 (with the head's and the squeeze-and-excite block's changes)
+// 1498 -> 790.
+constexpr int kDwC = 64;        // channels per block
+constexpr int kDwV = kDwC / 8;  // threads over them
+
+struct F8 {
+  float v[8];
+};
+__device__ __forceinline__ F8 up8(const uint4& u) {
+  const bf16* e = reinterpret_cast<const bf16*>(&u);
+  F8 r;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) r.v[j] = __bfloat162float(e[j]);
+  return r;
+}
+__device__ __forceinline__ F8 ld8(const bf16* p) { return up8(*reinterpret_cast<const uint4*>(p)); }
+__device__ __forceinline__ void st8(bf16* p, const F8& r) {
+  uint4 u;
+  bf16* e = reinterpret_cast<bf16*>(&u);
+#pragma unroll
+  for (int j = 0; j < 8; ++j) e[j] = __float2bfloat16_rn(r.v[j]);
+  *reinterpret_cast<uint4*>(p) = u;
+}
+__device__ __forceinline__ void fma8(F8& a, const F8& x, const float* w) {
+  const float4 w0 = *reinterpret_cast<const float4*>(w), w1 = *reinterpret_cast<const float4*>(w + 4);
+  a.v[0] = fmaf(x.v[0], w0.x, a.v[0]); a.v[1] = fmaf(x.v[1], w0.y, a.v[1]);
+  a.v[2] = fmaf(x.v[2], w0.z, a.v[2]); a.v[3] = fmaf(x.v[3], w0.w, a.v[3]);
+  a.v[4] = fmaf(x.v[4], w1.x, a.v[4]); a.v[5] = fmaf(x.v[5], w1.y, a.v[5]);
+  a.v[6] = fmaf(x.v[6], w1.z, a.v[6]); a.v[7] = fmaf(x.v[7], w1.w, a.v[7]);
+}
+
+// Block (channel block, pixel block of 16): DGRAD false, y = conv(x) + bias;
+// DGRAD true, y = dx (+)= conv^T(x = dy).  A tap outside the map loads the
+// first pixel and drops it, so that no branch keeps the loads of the taps
+// from being in flight together.
+constexpr int kDwThreads = 16 * kDwV;
+template <int KT, bool DGRAD>
+__global__ void __launch_bounds__(kDwThreads) dwconv_x8_k(const bf16* __restrict__ x, const bf16* __restrict__ w,
+                                                          const float* __restrict__ bias, bf16* __restrict__ y,
+                                                          DwShape d, unsigned rows, int acc_flag) {
+  pdl_wait();
+  pdl_trigger();
+  constexpr int KK = KT * KT;
+  __shared__ __align__(16) float ws[KK][kDwC + 4];
+  const int c0 = blockIdx.x * kDwC, nc = min(kDwC, d.C - c0);
+#pragma unroll 4
+  for (int e = threadIdx.x; e < nc * KK; e += kDwThreads)
+    ws[e % KK][e / KK] = __bfloat162float(w[int64_t(c0) * KK + e]);
+  __syncthreads();
+  const int cv = 8 * (threadIdx.x % kDwV), c = c0 + cv;
+  if (cv >= nc) return;
+  const unsigned Hy = DGRAD ? d.H : d.Ho, Wy = DGRAD ? d.W : d.Wo;   // the grid of y
+  const int Hx = DGRAD ? d.Ho : d.H, Wx = DGRAD ? d.Wo : d.W;        // the grid of x
+  for (unsigned p = blockIdx.y * 16 + threadIdx.x / kDwV; p < rows; p += gridDim.y * 16) {
+    const int j = int(p % Wy), i = int(p / Wy % Hy);
+    const bf16* xn = x + int64_t(p / (Wy * Hy)) * Hx * Wx * d.C + c;
+    F8 a;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) a.v[q] = !DGRAD && bias ? bias[c + q] : 0.f;
+#pragma unroll
+    for (int r = 0; r < KT; ++r) {
+      int h = DGRAD ? i + d.pad - r : i * d.stride - d.pad + r;
+      bool hok = h >= 0;
+      if (DGRAD && d.stride == 2) {
+        hok = hok && !(h & 1);
+        h >>= 1;
+      }
+      hok = hok && h < Hx;
+      uint4 u[KT];
+#pragma unroll
+      for (int s = 0; s < KT; ++s) {
+        int v = DGRAD ? j + d.pad - s : j * d.stride - d.pad + s;
+        bool ok = hok && v >= 0;
+        if (DGRAD && d.stride == 2) {
+          ok = ok && !(v & 1);
+          v >>= 1;
+        }
+        ok = ok && v < Wx;
+        const uint4 t = *reinterpret_cast<const uint4*>(xn + (ok ? int64_t(h * Wx + v) * d.C : 0));
+        u[s] = ok ? t : make_uint4(0u, 0u, 0u, 0u);
+      }
+#pragma unroll
+      for (int s = 0; s < KT; ++s) fma8(a, up8(u[s]), &ws[r * KT + s][cv]);
+    }
+    bf16* out = y + int64_t(p) * d.C + c;
+    if (acc_flag) {
+      const F8 o = ld8(out);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) a.v[q] += o.v[q];
+    }
+    st8(out, a);
+  }
+}
+
+// Weight (and bias) gradient partials of pixel chunk blockIdx.y, as
+// dwconv_wgrad_k: a thread takes 8 channels and one row of taps, and every
+// PL-th pixel of the chunk; the PL pixel lanes are added in order.
+template <int KT>
+__global__ void __launch_bounds__(240) dwconv_wgrad_x8_k(const bf16* __restrict__ dy, const bf16* __restrict__ x,
+                                                         float* __restrict__ pw, float* __restrict__ pb, DwShape d,
+                                                         unsigned rows, unsigned per) {
+  pdl_wait();
+  pdl_trigger();
+  constexpr int KK = KT * KT, PL = 240 / (kDwV * KT);
+  extern __shared__ float red[];   // [PL][KK + 1][kDwC + 1]
+  const int c0 = blockIdx.x * kDwC, nc = min(kDwC, d.C - c0);
+  const int cv = 8 * (threadIdx.x % kDwV), c = c0 + cv;
+  const int r = threadIdx.x / kDwV % KT, pl = threadIdx.x / (kDwV * KT);
+  const unsigned p0 = blockIdx.y * per, p1 = min(rows, p0 + per);
+  F8 a[KT], g;
+#pragma unroll
+  for (int s = 0; s < KT; ++s)
+#pragma unroll
+    for (int q = 0; q < 8; ++q) a[s].v[q] = 0.f;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) g.v[q] = 0.f;
+  if (cv < nc)
+    for (unsigned p = p0 + pl; p < p1; p += PL) {
+      const int j = int(p % unsigned(d.Wo)), i = int(p / unsigned(d.Wo) % unsigned(d.Ho));
+      const int64_t n = p / (unsigned(d.Wo) * unsigned(d.Ho));
+      const int h = i * d.stride - d.pad + r;
+      if (r > 0 && (h < 0 || h >= d.H)) continue;
+      const F8 dv = ld8(dy + int64_t(p) * d.C + c);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) g.v[q] += dv.v[q];
+      if (h < 0 || h >= d.H) continue;
+      const bf16* xr = x + (n * d.H + h) * int64_t(d.W) * d.C + c;
+      uint4 u[KT];
+#pragma unroll
+      for (int s = 0; s < KT; ++s) {   // a tap outside the row loads its first pixel and drops it
+        const int v = j * d.stride - d.pad + s;
+        const bool ok = v >= 0 && v < d.W;
+        const uint4 t = *reinterpret_cast<const uint4*>(xr + (ok ? int64_t(v) * d.C : 0));
+        u[s] = ok ? t : make_uint4(0u, 0u, 0u, 0u);
+      }
+#pragma unroll
+      for (int s = 0; s < KT; ++s) {
+        const F8 xv = up8(u[s]);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) a[s].v[q] = fmaf(dv.v[q], xv.v[q], a[s].v[q]);
+      }
+    }
+  float* mine = red + pl * (KK + 1) * (kDwC + 1) + cv;
+#pragma unroll
+  for (int s = 0; s < KT; ++s)
+#pragma unroll
+    for (int q = 0; q < 8; ++q) mine[(r * KT + s) * (kDwC + 1) + q] = a[s].v[q];
+  if (r == 0)   // row 0 saw every pixel: the bias sum
+#pragma unroll
+    for (int q = 0; q < 8; ++q) mine[KK * (kDwC + 1) + q] = g.v[q];
+  __syncthreads();
+  for (int e = threadIdx.x; e < nc * (KK + 1); e += 240) {
+    const int cl = e / (KK + 1), t = e % (KK + 1);
+    float sum = 0.f;
+#pragma unroll
+    for (int q = 0; q < PL; ++q) sum += red[(q * (KK + 1) + t) * (kDwC + 1) + cl];
+    if (t < KK) pw[int64_t(blockIdx.y) * d.C * KK + int64_t(c0 + cl) * KK + t] = sum;
+    else if (pb) pb[int64_t(blockIdx.y) * d.C + c0 + cl] = sum;
+  }
+}
+// 32-bit pixel indices, and 16-byte channel vectors.
+bool dw8_ok(const DwShape& d, int dt) {
+  return dt == kBF16 && d.C % 8 == 0 && (d.k == 3 || d.k == 5) && int64_t(d.N) * d.H * d.W < (int64_t(1) << 31);
+}
+
 int num_sms() {
   static int n = 0;
   if (n == 0) {
@@ -293,6 +465,13 @@ __global__ void chmul_bwd_k(const T* __restrict__ x, const T* __restrict__ sc, c
 
 void dwconv_fwd(const DwShape& d, const void* x, const void* w, const float* bias, void* y, int dt,
                 cudaStream_t st) {
+  if (dw8_ok(d, dt)) {
+    const unsigned rows = unsigned(d.N) * d.Ho * d.Wo;
+    const dim3 grid(ceil_div(d.C, kDwC), std::min(ceil_div(rows, 16), 65535));
+    launch_k(d.k == 3 ? dwconv_x8_k<3, false> : dwconv_x8_k<5, false>, grid, kDwThreads, 0, st, (const bf16*)x,
+             (const bf16*)w, bias, (bf16*)y, d, rows, 0);
+    return;
+  }
   const int64_t n = int64_t(d.N) * d.Ho * d.Wo * d.C;
   const int blocks = elementwise_blocks(n, 256);
   FO_MB_DISPATCH(dt, T, {
@@ -303,6 +482,13 @@ void dwconv_fwd(const DwShape& d, const void* x, const void* w, const float* bia
 }
 
 void dwconv_dgrad(const DwShape& d, const void* dy, const void* w, void* dx, int dt, bool acc, cudaStream_t st) {
+  if (dw8_ok(d, dt)) {
+    const unsigned rows = unsigned(d.N) * d.H * d.W;
+    const dim3 grid(ceil_div(d.C, kDwC), std::min(ceil_div(rows, 16), 65535));
+    launch_k(d.k == 3 ? dwconv_x8_k<3, true> : dwconv_x8_k<5, true>, grid, kDwThreads, 0, st, (const bf16*)dy,
+             (const bf16*)w, (const float*)nullptr, (bf16*)dx, d, rows, acc ? 1 : 0);
+    return;
+  }
   const int64_t n = int64_t(d.N) * d.H * d.W * d.C;
   const int blocks = elementwise_blocks(n, 256);
   const int a = acc ? 1 : 0;
@@ -336,6 +522,13 @@ void dwconv_wgrad_pass(const DwShape& d, const void* dy, const void* x, int dt, 
   const int64_t rows = int64_t(d.N) * d.Ho * d.Wo;
   const int chunks = dwconv_wgrad_chunks(d);
   const int per = int((rows + chunks - 1) / chunks);
+  if (dw8_ok(d, dt)) {
+    const dim3 grid(ceil_div(d.C, kDwC), chunks);
+    const size_t sm = sizeof(float) * (240 / (kDwV * d.k)) * (d.k * d.k + 1) * (kDwC + 1);   // below 48 KB
+    launch_k(d.k == 3 ? dwconv_wgrad_x8_k<3> : dwconv_wgrad_x8_k<5>, grid, 240, sm, st, (const bf16*)dy,
+             (const bf16*)x, pw, pb, d, unsigned(rows), unsigned(per));
+    return;
+  }
   if (d.k == 3 || d.k == 5) {
     dim3 grid(ceil_div(d.C, 32), chunks);
     FO_MB_DISPATCH(dt, T, {
