@@ -11,6 +11,7 @@
 #include <memory>
 #include "fo_tc.h"
 
+#include <array>
 #include <cstring>
 #include <functional>
 #include <map>
@@ -222,6 +223,9 @@ struct Fusion {
   // A linear layer whose output feeds only a GELU: its epilogue may store
   // the GELU too (the plan decides; the GELU op runs alone otherwise).
   std::vector<int> gelu_of;    // producer op -> the GELU op, or -1
+  // Residual add whose operand is an affine's output that nothing else reads:
+  // the add forms it on the fly (its backward needs only the add's mask).
+  std::vector<std::array<int, 2>> add_affine;   // add op -> per operand (in0, in1): the affine op, or -1
   bool head = false;           // last linear + loss handled by the head kernels
 };
 
@@ -310,6 +314,20 @@ Fusion analyse(const fo_server* s) {
       f.branch_of[a] = t;
       f.skip_fwd[a] = 1;
       break;
+    }
+  }
+  f.add_affine.assign(nops, {-1, -1});
+  for (int a = 0; a < nops; ++a) {
+    const fo_op& op = s->ops[a];
+    if (op.kind != FO_OP_ADD || f.branch_of[a] >= 0 || !fo::vec8_ok(s->dt, s->T[a + 1].numel()) || s->T[a + 1].C % 8)
+      continue;
+    const int in[2] = {op.in0, op.in1};
+    for (int q = 0; q < 2; ++q) {
+      if (s->T[in[q]].is_input() || sole[in[q]] != a) continue;
+      const int p = in[q] - 1;
+      if (s->ops[p].kind != FO_OP_AFFINE || f.fwd_relu[p] >= 0 || f.hswish_of[p] >= 0) continue;
+      f.add_affine[a][q] = p;
+      f.skip_fwd[p] = 1;
     }
   }
   for (int g = 0; g < nops && !getenv("FO_NO_GELU_EPILOGUE"); ++g) {
@@ -468,6 +486,17 @@ int build_plan(fo_server* s) {
         break;
       case FO_OP_ADD: {
         const int b = op.in1;
+        const int p0 = fu.add_affine[i][0], p1 = fu.add_affine[i][1];
+        if (p0 >= 0 || p1 >= 0) {
+          const int pa = p0 >= 0 ? p0 : p1;                    // the first operand's affine
+          const int pb = p0 >= 0 ? p1 : -1;                    // the second's, if it has one
+          const int xa = s->ops[pa].in0, xb = pb >= 0 ? s->ops[pb].in0 : (p0 >= 0 ? b : a);
+          add("affine_add_fwd", 1, 0.0, 3 * tbytes(i + 1), [=](cudaStream_t st) {
+            fo::affine_add_x8(act(xa), P(s, pa, 0), P(s, pa, 1), act(xb), pb >= 0 ? P(s, pb, 0) : nullptr,
+                              pb >= 0 ? P(s, pb, 1) : nullptr, s->T[o].act, s->T[o].numel(), s->T[o].C, relu, st);
+          });
+          break;
+        }
         add("add_fwd", 1, 0.0, 3 * tbytes(i + 1), [=](cudaStream_t st) {
           fo::add_fwd(act(a), act(b), s->T[o].act, s->T[o].numel(), dt, relu, st);
         });

@@ -380,10 +380,75 @@ __global__ void avgpool_bwd_k(const T* dy, T* dx, int N, int HW, int C, int acc)
     store(dx, i, to_f(dy[n * C + c]) / float(HW), acc);
   }
 }
+// 8 channels per thread (bf16, C % 8 == 0).  A block takes an image and GL
+// channel vectors, its 256 / GL pixel lanes take every so-many-th pixel and
+// are added in lane order: one thread per (image, channel) walked the pixels
+// alone, in 32 blocks for 64 images of 16 x 16 x 128 (24.4 us alone).  A device
+// trainer's step went from 177 to 161 us with both passes.
+__global__ void __launch_bounds__(256) avgpool_fwd_x8_k(const bf16* __restrict__ x, bf16* __restrict__ y, int HW, int C,
+                                                        int GL) {
+  pdl_wait();
+  pdl_trigger();
+  __shared__ float red[256][9];
+  const int PL = 256 / GL, g = threadIdx.x % GL, pl = threadIdx.x / GL;
+  const int c = (blockIdx.y * GL + g) * 8;
+  float sum[8] = {};
+  if (c < C) {
+    const bf16* base = x + int64_t(blockIdx.x) * HW * C + c;
+#pragma unroll 4
+    for (int p = pl; p < HW; p += PL) {
+      const uint4 u = *reinterpret_cast<const uint4*>(base + int64_t(p) * C);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) sum[j] += to_f(reinterpret_cast<const bf16*>(&u)[j]);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) red[threadIdx.x][j] = sum[j];
+  __syncthreads();
+  for (int e = threadIdx.x; e < GL * 8; e += 256) {
+    const int cc = blockIdx.y * GL * 8 + e;
+    if (cc >= C) break;
+    float t = 0.f;
+    for (int q = 0; q < PL; ++q) t += red[q * GL + e / 8][e % 8];
+    y[int64_t(blockIdx.x) * C + cc] = from_f<bf16>(t / float(HW));
+  }
+}
+__global__ void __launch_bounds__(256) avgpool_bwd_x8_k(const bf16* __restrict__ dy, bf16* __restrict__ dx, unsigned n8,
+                                                        unsigned C8, unsigned HW, int acc) {
+  pdl_wait();
+  pdl_trigger();
+  const float hw = float(HW);
+  for (unsigned i = blockIdx.x * 256u + threadIdx.x; i < n8; i += gridDim.x * 256u) {
+    const unsigned c8 = i % C8, n = i / C8 / HW;
+    const uint4 u = *reinterpret_cast<const uint4*>(dy + 8 * (int64_t(n) * C8 + c8));
+    uint4 o = make_uint4(0u, 0u, 0u, 0u);
+    if (acc) o = *reinterpret_cast<const uint4*>(dx + 8 * int64_t(i));
+    bf16* ob = reinterpret_cast<bf16*>(&o);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      float v = to_f(reinterpret_cast<const bf16*>(&u)[j]) / hw;
+      if (acc) v += to_f(ob[j]);
+      ob[j] = from_f<bf16>(v);
+    }
+    *reinterpret_cast<uint4*>(dx + 8 * int64_t(i)) = o;
+  }
+}
 void avgpool_fwd(const void* x, void* y, int N, int HW, int C, int dt, cudaStream_t st) {
+  if (dt == kBF16 && C % 8 == 0) {
+    int GL = 4;   // channel vectors per block: the fewest blocks' worth that covers C, at most a warp's
+    while (GL < 32 && GL * 8 < C) GL *= 2;
+    launch_k(avgpool_fwd_x8_k, dim3(N, ceil_div(C, GL * 8)), 256, 0, st, (const bf16*)x, (bf16*)y, HW, C, GL);
+    return;
+  }
   FO_DISPATCH(dt, T, launch_k(avgpool_fwd_k<T>, elementwise_blocks(int64_t(N) * C, 256), 256, 0, st, (const T*)x, (T*)y, N, HW, C));
 }
 void avgpool_bwd(const void* dy, void* dx, int N, int HW, int C, int dt, bool acc, cudaStream_t st) {
+  const int64_t n8 = int64_t(N) * HW * C / 8;
+  if (dt == kBF16 && C % 8 == 0 && n8 < (int64_t(1) << 31)) {   // 32-bit vector indices (the stride adds less than 2^19)
+    launch_k(avgpool_bwd_x8_k, elementwise_blocks(n8, 256), 256, 0, st, (const bf16*)dy, (bf16*)dx, unsigned(n8),
+             unsigned(C / 8), unsigned(HW), acc ? 1 : 0);
+    return;
+  }
   FO_DISPATCH(dt, T, launch_k(avgpool_bwd_k<T>, elementwise_blocks(int64_t(N) * HW * C, 256), 256, 0, st, (const T*)dy, (T*)dx, N, HW, C, acc));
 }
 
