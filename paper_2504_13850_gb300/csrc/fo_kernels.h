@@ -99,9 +99,10 @@ void head_forward_loss(const void* x, int dt, const float* W, const float* bias,
                        int B, int K, int C, float* logits, float* dz, float* row_loss, cudaStream_t st,
                        const void* mask = nullptr, void* dx = nullptr, bool acc = false);
 // The batch loss goes to losses[*step & mask].
+// mirror (may be null): a second ring that gets the loss, indexed with mirror_mask.
 void head_weight_grad(const float* dz, const void* x, int dt, int B, int K, int C, float* dW, float* db,
                       const float* row_loss, float* losses, const int64_t* step, int64_t mask,
-                      cudaStream_t st);
+                      cudaStream_t st, float* mirror = nullptr, int64_t mirror_mask = 0);
 
 // Softmax cross-entropy: losses[*step & mask] <- mean_b CE; dlogits = (softmax - onehot)/B.
 void softmax_ce(const float* logits, const int32_t* labels, int B, int C, float* losses,
@@ -198,6 +199,11 @@ void layernorm_bwd8_pass(const void* x, const float* gamma, const float* mean, c
                          void* dx, int64_t rows, int C, bool acc, float* p_gamma, float* p_beta, cudaStream_t st,
                          const void* addend = nullptr, float* p_dx = nullptr);
 
+
+// One upload from device memory: `bytes` of activations (src 16-byte aligned)
+// and B labels and, when given, lengths.
+void upload_copy(const void* acts, void* d_acts, int64_t bytes, const int32_t* labels, int32_t* d_labels,
+                 const int32_t* lengths, int32_t* d_lengths, int B, cudaStream_t st);
 
 // ---- MobileNetV3 bottleneck (k_mobile.cu) ----
 // Depthwise k x k convolution, NHWC, weights [C][k][k] in the activation

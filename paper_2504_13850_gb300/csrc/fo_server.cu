@@ -368,6 +368,7 @@ int build_plan(fo_server* s) {
     add(fo::tc_name(g), 1, fo::tc_flops(g), 0.0, [=](cudaStream_t st) { fo::tc_run(g, nullptr, st); }, lane);
   };
   const int L = nops - 1;  // the logits layer
+  s->loss_mirrored = fu.head;
 
   // Max-pools computed by the epilogue of the conv / linear in front of them
   // (through its ReLU): per pool op, the window codes that epilogue stores,
@@ -704,7 +705,7 @@ int build_plan(fo_server* s) {
       add("head_wgrad", 1, 2.0 * B * K * C, tbytes(a0), [=](cudaStream_t st) {
         fo::head_weight_grad((const float*)s->T[o].grad, act(a0), s->T[a0].dt, B, K, C, G(s, i, 0),
                              op.bias ? G(s, i, 1) : nullptr, s->row_loss, s->losses, s->d_step,
-                             s->kLossRing - 1, st);
+                             s->kLossRing - 1, st, s->loss_host_dev, s->kLossMirror - 1);
       }, 1);
       if (need_dx && contrib(a) != 0)   // formed in the forward launch as the first contribution
         return set_err(FO_ERR_ARG, "classifier input gradient is not the first contribution");
@@ -1215,6 +1216,8 @@ int allocate(fo_server* s) {
   s->use_graphs = getenv("FO_NO_GRAPH") == nullptr;
   if (!s->colsum_scratch || !s->losses) return set_err(FO_ERR_OOM, "scratch allocation");
   FO_CUDA(cudaMemset(s->losses, 0, size_t(s->kLossRing) * 4));
+  FO_CUDA(cudaHostAlloc((void**)&s->loss_host, size_t(s->kLossMirror) * 4, cudaHostAllocMapped | cudaHostAllocPortable));
+  FO_CUDA(cudaHostGetDevicePointer((void**)&s->loss_host_dev, s->loss_host, 0));
   return FO_OK;
 }
 
@@ -1245,6 +1248,7 @@ void destroy_impl(fo_server* s) {
   if (s->side) cudaStreamSynchronize(s->side);
   if (s->opt_st) cudaStreamSynchronize(s->opt_st);
   for (void* p : s->allocs) cudaFree(p);
+  if (s->loss_host) cudaFreeHost(s->loss_host);
   for (int b = 0; b < 2; ++b) {
     if (s->agg_stage[b]) cudaFree(s->agg_stage[b]);
     if (s->agg_landed[b]) cudaEventDestroy(s->agg_landed[b]);
@@ -1498,6 +1502,17 @@ int fo_server_store_params_device(fo_server* s, float* dst, int64_t n) {
   return FO_OK;
 }
 
+// True for memory of the current device at a multiple of `align` bytes, which a kernel may read.
+static bool on_device(const void* p, uintptr_t align) {
+  cudaPointerAttributes a{};
+  int dev = -1;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == dev && reinterpret_cast<uintptr_t>(p) % align == 0;
+}
+
 // The copies of an accepted upload into batch slot `slot` (before the
 // scheduler commits it).
 static int upload_copies(fo_server* s, int32_t slot, const void* acts, const int32_t* labels,
@@ -1511,6 +1526,13 @@ static int upload_copies(fo_server* s, int32_t slot, const void* acts, const int
     const cudaError_t q = cudaEventQuery(s->slot_free[slot]);
     if (q == cudaErrorNotReady) busy = true;
     else FO_CUDA(q);
+  }
+  if (!busy && on_device(acts, 16) && on_device(labels, 4) && (!lengths || on_device(lengths, 4))) {
+    fo::upload_copy(acts, d_act, s->slot_act_bytes, labels, d_lab, lengths, d_len, B, s->hs);
+    FO_CUDA(cudaGetLastError());
+    FO_CUDA(cudaEventRecord(s->slot_ready[slot], s->hs));
+    FO_CUDA(cudaEventSynchronize(s->slot_ready[slot]));   // the caller may reuse its buffers
+    return FO_OK;
   }
   if (!busy) {
     FO_CUDA(cudaMemcpyAsync(d_act, acts, s->slot_act_bytes, cudaMemcpyDefault, s->hs));
@@ -1663,8 +1685,12 @@ int fo_read_losses(fo_server* s, float* host_out, int64_t first_step, int64_t n)
   // either way the losses asked for are written once it has completed.
   FO_CUDA(cudaEventSynchronize(s->step_done[(first_step + n - 1) % fo_server::kStepEvents]));
   for (int64_t i = 0; i < n; ++i) {
-    int64_t idx = (first_step + i) & (s->kLossRing - 1);
-    FO_CUDA(cudaMemcpy(host_out + i, s->losses + idx, 4, cudaMemcpyDeviceToHost));
+    const int64_t step = first_step + i;
+    if (s->loss_mirrored && s->steps_done - step <= s->kLossMirror) {   // no step issued since reuses its place
+      host_out[i] = static_cast<volatile float*>(s->loss_host)[step & (s->kLossMirror - 1)];
+      continue;
+    }
+    FO_CUDA(cudaMemcpy(host_out + i, s->losses + (step & (s->kLossRing - 1)), 4, cudaMemcpyDeviceToHost));
   }
   return FO_OK;
 }

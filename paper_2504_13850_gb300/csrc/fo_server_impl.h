@@ -119,6 +119,12 @@ struct fo_server {
   const int32_t* cur_labels = nullptr;
   const int32_t* cur_len = nullptr;
   float* losses = nullptr;
+  // The newest kLossMirror losses again, in page-locked host memory that the
+  // classifier's kernel writes: reading a step's loss needs no copy.
+  static constexpr int64_t kLossMirror = 1024;
+  float* loss_host = nullptr;       // host address
+  float* loss_host_dev = nullptr;   // the same memory for the device
+  bool loss_mirrored = false;       // the plan's loss kernel writes it
   float* row_loss = nullptr;
   int64_t* d_step = nullptr;   // device copy of steps_done (indexes the loss ring)
   bool use_graphs = true;

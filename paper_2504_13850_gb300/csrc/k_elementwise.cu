@@ -357,6 +357,40 @@ void add_fwd(const void* a, const void* b, void* y, int64_t n, int dt, bool relu
   FO_DISPATCH(dt, T, launch_k(add_fwd_k<T>, elementwise_blocks(n, 256), 256, 0, st, (const T*)a, (const T*)b, (T*)y, n, relu));
 }
 
+// --------------------------------------------------------------- upload
+// A batch that is in device memory already: activations, labels and lengths in
+// one launch (as three stream copies each had its own start, and the caller
+// waits for the last one).
+__global__ void __launch_bounds__(256) upload_copy_k(const uint4* __restrict__ a, uint4* __restrict__ da, int64_t n16,
+                                                     const char* __restrict__ tail, char* __restrict__ dtail, int nt,
+                                                     const int32_t* __restrict__ lab, int32_t* __restrict__ dlab,
+                                                     const int32_t* __restrict__ len, int32_t* __restrict__ dlen, int B) {
+  const int64_t step = int64_t(gridDim.x) * 256;
+  int64_t i = int64_t(blockIdx.x) * 256 + threadIdx.x;
+  if (i < nt) dtail[i] = tail[i];
+  if (i < B) {
+    dlab[i] = lab[i];
+    if (len) dlen[i] = len[i];
+  }
+  for (; i + 3 * step < n16; i += 4 * step) {   // four loads in flight
+    const uint4 u0 = a[i], u1 = a[i + step], u2 = a[i + 2 * step], u3 = a[i + 3 * step];
+    da[i] = u0;
+    da[i + step] = u1;
+    da[i + 2 * step] = u2;
+    da[i + 3 * step] = u3;
+  }
+  for (; i < n16; i += step) da[i] = a[i];
+}
+void upload_copy(const void* acts, void* d_acts, int64_t bytes, const int32_t* labels, int32_t* d_labels,
+                 const int32_t* lengths, int32_t* d_lengths, int B, cudaStream_t st) {
+  const int64_t n16 = bytes / 16;
+  const int nt = int(bytes % 16);
+  // at least one thread per label (B <= 1024) and tail byte
+  const int blocks = elementwise_blocks(std::max<int64_t>(n16 / 4, std::max(B, 16)), 256);
+  upload_copy_k<<<blocks, 256, 0, st>>>((const uint4*)acts, (uint4*)d_acts, n16, (const char*)acts + 16 * n16,
+                                        (char*)d_acts + 16 * n16, nt, labels, d_labels, lengths, d_lengths, B);
+}
+
 // -------------------------------------------------------------- avgpool
 template <typename T>
 __global__ void avgpool_fwd_k(const T* x, T* y, int N, int HW, int C) {

@@ -235,7 +235,8 @@ __global__ void __launch_bounds__(kHeadThreads) head_fwd_ce_k(
 template <typename T>
 __global__ void head_wgrad_k(const float* __restrict__ dz, const T* __restrict__ x, int B, int K, int C,
                              float* __restrict__ dW, float* __restrict__ db, const float* __restrict__ row_loss,
-                             float* __restrict__ losses, const int64_t* __restrict__ step, int64_t mask) {
+                             float* __restrict__ losses, const int64_t* __restrict__ step, int64_t mask,
+                             float* __restrict__ mirror, int64_t mirror_mask) {
   pdl_wait();
   pdl_trigger();
   __shared__ float xs[64][33];
@@ -271,6 +272,7 @@ __global__ void head_wgrad_k(const float* __restrict__ dz, const T* __restrict__
 #pragma unroll 8
       for (int b = 0; b < B; ++b) t += rl[b];
       losses[*step & mask] = t / float(B);
+      if (mirror) mirror[*step & mirror_mask] = t / float(B);
     }
   }
 }
@@ -326,12 +328,14 @@ void head_forward_loss(const void* x, int dt, const float* W, const float* bias,
 
 void head_weight_grad(const float* dz, const void* x, int dt, int B, int K, int C, float* dW, float* db,
                       const float* row_loss, float* losses, const int64_t* step, int64_t mask,
-                      cudaStream_t st) {
+                      cudaStream_t st, float* mirror, int64_t mirror_mask) {
   dim3 grid(ceil_div(K, 32), ceil_div(C, 8));
   if (dt == kF32)
-    launch_k(head_wgrad_k<float>, grid, 256, 0, st, dz, (const float*)x, B, K, C, dW, db, row_loss, losses, step, mask);
+    launch_k(head_wgrad_k<float>, grid, 256, 0, st, dz, (const float*)x, B, K, C, dW, db, row_loss, losses, step, mask, mirror,
+             mirror_mask);
   else
-    launch_k(head_wgrad_k<bf16>, grid, 256, 0, st, dz, (const bf16*)x, B, K, C, dW, db, row_loss, losses, step, mask);
+    launch_k(head_wgrad_k<bf16>, grid, 256, 0, st, dz, (const bf16*)x, B, K, C, dW, db, row_loss, losses, step, mask, mirror,
+             mirror_mask);
 }
 
 }  // namespace fo
