@@ -216,7 +216,7 @@ bool window_ok(int H, int W, int rows_needed, int* rows, int* imgs) {
 // stride x stride patch of the input.  Where either rule fails (7, 14 or 28
 // pixel rows, odd maps) the window is loaded in im2col mode; such layers ran
 // on the CUDA-core kernel before (bf16, 5-9 TFLOP/s against 200-240 here):
-// ResNet-18 stages 3-4 on 28 x 28 maps at batch 24, 20.6 -> 0.72 ms a step;
+// ResNet-18 stages 3-4 on 28 x 28 maps at batch 24, 20.6 -> 0.72 ms a step then;
 // the VGG part at batch 37, whose last tile is partial, 8.0 -> 0.26 ms.
 bool whole_windows(const fo_op& op, const Tensor& a, const Tensor& o) {
   return op.stride == 1 || (a.H == 2 * o.H && a.W == 2 * o.W);
@@ -264,6 +264,12 @@ int active_clusters(TcContext* c, int kind, int bn, int S, int epi) {
 //    whole steps (us; these / 0.37, 0.37, 0.375 / 0.21, 0.24, 0.36): VGG 270 /
 //    269 / 271, ResNet 540 / 544 / 532, ResNet on 28 x 28 maps 643 / 662 / 660,
 //    transformer 741 / 756 / 775, one narrow ragged block 269 / 278 / 289;
+//  * a launch that leaves SMs to others is charged the uncontended stage (0.21
+//    / 0.24 / 0.34): plain GEMMs on up to half of the SMs, tiled convolutions
+//    up to 0.85 of them, im2col windows never.  Whole steps with these limits
+//    at 0 / 0.5 / 0.85 for all kinds: ResNet 464 / 456 / 447, VGG 255 / 256 /
+//    253, one 384-wide encoder block 156 / 151 / 157, transformer 726 / 728 /
+//    755, ResNet on 28 x 28 maps 429 / 438 / 435;
 //  * a CTA pays a start-up ramp and the epilogue of its last tile (earlier
 //    epilogues overlap the next tile's MMAs), a K-split cluster pays the
 //    exchange of its partial tiles through the L2 workspace and their
@@ -285,8 +291,9 @@ void choose_tiles(TcContext* c, TcGemm* g, int M, int N, int KB, int ndiv) {
     const int n_tiles = (N + bn - 1) / bn, m_tiles = (M + BM - 1) / BM, tiles = n_tiles * m_tiles;
     const double epi = bn == 256 ? 4.2 : (bn == 128 ? 2.2 : 1.5);
     const bool mn = g->kind == LIN_WGRAD || win_b;
-    double t_kb = (bn == 256 ? 0.375 : (bn == 128 ? 0.32 : 0.30)) + (mn ? 0.015 : 0.0);
-    if (win_b && g->p.im2col) t_kb = std::max(t_kb, 0.1 + 0.1 * bn / 64);   // one box per 64 channels
+    const double t_busy = (bn == 256 ? 0.375 : (bn == 128 ? 0.32 : 0.30)) + (mn ? 0.015 : 0.0);
+    const double t_alone = (bn == 256 ? 0.34 : (bn == 128 ? 0.24 : 0.21)) + (mn ? 0.015 : 0.0);
+    const double alone = g->p.im2col ? 0.0 : (win_a || win_b ? 0.85 : 0.5);   // share of the SMs up to which it applies
     for (int sp = 1; sp <= 8; ++sp) {
       if (sp > 1 && KB / sp < 4) break;
       // an owner's receive slices (16 KB per other rank and owned chunk) live in the pipeline buffers
@@ -294,6 +301,8 @@ void choose_tiles(TcContext* c, TcGemm* g, int M, int N, int KB, int ndiv) {
       const int kper = (KB + sp - 1) / sp;
       const int splits = (KB + kper - 1) / kper;
       if (splits != sp) continue;
+      double t_kb = tiles * splits <= alone * c->num_sms ? t_alone : t_busy;
+      if (win_b && g->p.im2col) t_kb = std::max(t_kb, 0.1 + 0.1 * bn / 64);   // one box per 64 channels
       double cost;
       if (splits == 1) {
         const int units = std::min(tiles, c->num_sms);
