@@ -13,12 +13,16 @@
 // columns wide: a narrower head's tile goes on into its neighbour's columns
 // (or zeros past the last), which the products over DH never read and whose
 // output columns are not stored.
-// Narrower heads multiply P and dS as the sum of two bf16 tiles (value and
-// remainder, 16 bits of mantissa; SPLIT), since those widths ran in fp32 on
-// the CUDA cores before; their products then cost twice the MMAs of a path
-// that waits on latency, not on the tensor pipe.  One 256-wide encoder block of
-// 19 x 77 tokens, 8 heads of 32: the CUDA-core kernels took 36.7 us forward and
-// 61.4 backward alone; the whole step went from 279 to 143 us.
+// Narrower heads keep P and dS in fp32 (SPLIT): a value is multiplied as the
+// sum of three bf16 terms, value, remainder and remainder of that, whose 8-bit
+// mantissas hold all 24 bits, and each product with a bf16 operand is exact in
+// the fp32 accumulator.  The backward then has room for one of P and dS at a
+// time: dV = P^T dO first, then dS takes P's tiles.  Two terms (16 bits) were
+// not enough: 0.17-0.26% of the outputs and gradients differed from the exact
+// value rounded to bf16, against 0.01-0.04% on the fp32 CUDA-core kernels
+// that these widths ran on before.  A step of one 256-wide encoder block of
+// 19 x 77 tokens, 8 heads of 32: 289 us with those, 127 with two terms, 131
+// with three (64 x 128 tokens: 223 with two, 240 with three).
 // Operand tiles are 128 rows x 64 bf16 (128-byte rows, 128-byte swizzle),
 // loaded by TMA from the packed q|k|v [B*L, 3C] and dO [B*L, C] (the
 // backward reads O's rows directly for rowsum(dO * O));
@@ -30,7 +34,7 @@
 // reads TMEM lane quarter w % 4 (32 rows) and takes keys 64 * ((w - 2) / 4)
 // .. +63 of them, so every row is shared by two threads (the forward pass
 // combines their partial maxima and sums through shared memory).  Waits are
-// bounded (error word 11..16).
+// bounded (error word 11..17).
 #include "fo_common.cuh"
 #include "fo_kernels.h"
 #include "fo_ptx.cuh"
@@ -66,22 +70,26 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
-// v[0..8) as bf16 into a tile's 16-byte unit at `hi` and, when SPLIT, the
-// remainders of that rounding at `lo`.
-template <bool SPLIT>
-__device__ __forceinline__ void st_unit(uint32_t hi, uint32_t lo, const float (&v)[8]) {
-  uint32_t h[4];
+// Byte offset of term t's tiles from those of term 0 (SPLIT, both passes).
+__host__ __device__ constexpr uint32_t term_off(int t) { return t ? uint32_t(2 * t + 1) * kTile : 0u; }
+
+// v[0..8) as a sum of TERMS bf16 values, term t into the 16-byte unit at
+// at + term_off(t).  A term that overflows to infinity has no remainder.
+template <int TERMS>
+__device__ __forceinline__ void st_unit(uint32_t at, float (&v)[8]) {
 #pragma unroll
-  for (int q = 0; q < 4; ++q) h[q] = pack_bf16x2(v[2 * q], v[2 * q + 1]);
-  st_shared4(hi, h[0], h[1], h[2], h[3]);
-  if constexpr (SPLIT) {
-    uint32_t l[4];
+  for (int t = 0; t < TERMS; ++t) {
+    uint32_t h[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const __nv_bfloat162 b = *reinterpret_cast<const __nv_bfloat162*>(&h[q]);
-      l[q] = pack_bf16x2(v[2 * q] - __low2float(b), v[2 * q + 1] - __high2float(b));
+      h[q] = pack_bf16x2(v[2 * q], v[2 * q + 1]);
+      if (t + 1 < TERMS) {
+        const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h[q]));
+        v[2 * q] = isinf(f.x) ? 0.f : v[2 * q] - f.x;
+        v[2 * q + 1] = isinf(f.y) ? 0.f : v[2 * q + 1] - f.y;
+      }
     }
-    st_shared4(lo, l[0], l[1], l[2], l[3]);
+    st_shared4(at + term_off(t), h[0], h[1], h[2], h[3]);
   }
 }
 
@@ -126,14 +134,20 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_fwd_tc_k(const __grid_co
   char* sQ = sm;
   char* sK = sm + kTile;
   char* sV = sm + 2 * kTile;
-  // P~: two sub-tiles (keys 0..63, 64..127); SPLIT: the values over Q and K,
-  // which S = Q K^T alone reads, and the remainders in the two tiles after V
+  // P~: two sub-tiles (keys 0..63, 64..127); SPLIT: the first term over Q and
+  // K, which S = Q K^T alone reads, the others in the tiles after V
+  constexpr int kTerms = SPLIT ? 3 : 1;
   char* sP = SPLIT ? sm : sm + 3 * kTile;
-  char* sPlo = sm + 3 * kTile;
   const float kScale = attn_scale<DH>();
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sm + 5 * kTile);   // ld, s, p, o
+  // barriers (ld, s, p, o) and the TMEM slot; SPLIT: as in the backward pass
+  uint64_t* bars = reinterpret_cast<uint64_t*>(!SPLIT ? sm + 5 * kTile : (sm - smem_raw >= 64 ? smem_raw : sm + 7 * kTile));
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 4);
-  float2* xch = reinterpret_cast<float2*>(sm + 5 * kTile + 64);   // [half][row]: partial maxima, then sums
+  // [half][row]: partial maxima, then sums; SPLIT: in the last unit of V's
+  // rows, whose columns no head this narrow has
+  auto xch = [&](int half, int row, int sum) -> float* {
+    if (SPLIT) return reinterpret_cast<float*>(sV + sw_off(row, 7)) + 2 * sum + half;
+    return reinterpret_cast<float*>(sm + 5 * kTile + 64) + (2 * sum + half) * 128 + row;
+  };
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int bh = blockIdx.x, b = bh / p.heads, h = bh % p.heads;
@@ -180,14 +194,11 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_fwd_tc_k(const __grid_co
       tc_fence_after();
       constexpr uint32_t id_o = instr_desc(64, false, true);
 #pragma unroll
-      for (int k = 0; k < 8; ++k)
-        mma_f16(tmem + 128, smem_desc(smem_u32(sP) + (k >> 2) * kTile + 32 * (k & 3), 16, 1024),
-                smem_desc(smem_u32(sV) + 2048 * k, kTile, 1024), id_o, k > 0 ? 1u : 0u);
-      if constexpr (SPLIT)
+      for (int t = 0; t < kTerms; ++t)
 #pragma unroll
         for (int k = 0; k < 8; ++k)
-          mma_f16(tmem + 128, smem_desc(smem_u32(sPlo) + (k >> 2) * kTile + 32 * (k & 3), 16, 1024),
-                  smem_desc(smem_u32(sV) + 2048 * k, kTile, 1024), id_o, 1u);
+          mma_f16(tmem + 128, smem_desc(smem_u32(sP) + term_off(t) + (k >> 2) * kTile + 32 * (k & 3), 16, 1024),
+                  smem_desc(smem_u32(sV) + 2048 * k, kTile, 1024), id_o, t + k > 0 ? 1u : 0u);
       mma_commit(&bars[3]);
     }
   } else {
@@ -207,14 +218,13 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_fwd_tc_k(const __grid_co
       for (int e = 0; e < 32; ++e)
         if (j0 + e < n) m = fmaxf(m, __uint_as_float(r[e]) * kScale);
     }
-    xch[hf * 128 + i] = make_float2(m, 0.f);
+    *xch(hf, i, 0) = m;
     asm volatile("bar.sync 1, %0;" ::"n"(kSoftmaxThreads) : "memory");
-    const float M = fmaxf(m, xch[(1 - hf) * 128 + i].x);
+    const float M = fmaxf(m, *xch(1 - hf, i, 0));
     // P~ = exp(s / 8 - M) (bf16, unnormalised: one exponential per score) and
     // its row sum; O = P~ V is normalised by the sum in the store below
     float sum = 0.f;
     const uint32_t p_base = smem_u32(sP) + uint32_t(hf) * kTile;
-    const uint32_t l_base = smem_u32(sPlo) + uint32_t(hf) * kTile;
 #pragma unroll 1
     for (int c = 0; c < 2; ++c) {
       tmem_ld32(trow + 32 * c, r);
@@ -227,16 +237,16 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_fwd_tc_k(const __grid_co
           v[e] = j < n ? attn_exp<SPLIT>(__uint_as_float(r[8 * g + e]) * kScale - M) : 0.f;
           sum += v[e];
         }
-        st_unit<SPLIT>(p_base + sw_off(i, c * 4 + g), l_base + sw_off(i, c * 4 + g), v);
+        st_unit<kTerms>(p_base + sw_off(i, c * 4 + g), v);
       }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // P~ visible to the tensor cores
     tc_fence_before();
     mbar_arrive(&bars[2]);
     // the row sum over both halves, while the tensor cores form O
-    xch[256 + hf * 128 + i] = make_float2(sum, 0.f);
+    *xch(hf, i, 1) = sum;
     asm volatile("bar.sync 1, %0;" ::"n"(kSoftmaxThreads) : "memory");
-    const float S = sum + xch[256 + (1 - hf) * 128 + i].x;
+    const float S = sum + *xch(1 - hf, i, 1);
     const float inv = S > 0.f ? 1.f / S : 0.f;
     if (hf == 0 && i < p.L) p.lse[size_t(bh) * p.L + i] = M + logf(S);
     if (!mbar_wait(&bars[3], 0)) atomicExch(p.err, 14);
@@ -260,7 +270,8 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_fwd_tc_k(const __grid_co
 // buffer once that phase has completed; O is read from global memory (only
 // its row sums with dO are needed); dQ, dV and dK take the TMEM columns of S
 // and dP, which the softmax warps have read before the second phase starts.
-// SPLIT: four more tiles hold the remainders of P and dS, one CTA per SM.
+// SPLIT: 9 tiles, one CTA per SM: the other two terms of P take four more, and
+// the terms of dS, held in registers until dV is formed, take those of P.
 template <int DH, bool SPLIT>
 __global__ void __launch_bounds__(kAttnThreads, SPLIT ? 1 : 2) attn_bwd_tc_k(const __grid_constant__ AttnParams p) {
   extern __shared__ __align__(1024) char smem_raw[];
@@ -270,15 +281,15 @@ __global__ void __launch_bounds__(kAttnThreads, SPLIT ? 1 : 2) attn_bwd_tc_k(con
   char* sV = sm + 2 * kTile;
   char* sP = sm + 2 * kTile;      // two sub-tiles: V's buffer after the first phase, then the next
   char* sdO = sm + 4 * kTile;
-  char* sdS = sm + 5 * kTile;     // two sub-tiles
-  char* sPlo = sm + 7 * kTile;    // SPLIT: two sub-tiles each
-  char* sdSlo = sm + 9 * kTile;
+  char* sdS = SPLIT ? sP : sm + 5 * kTile;   // two sub-tiles
+  constexpr int kTerms = SPLIT ? 3 : 1;
   const float kScale = attn_scale<DH>();
-  // barriers (ld, s, p, g) and the TMEM slot: in the alignment slack below
-  // the tiles when it has room, else after them (the request covers both)
+  // barriers (ld, s, p, g and, SPLIT, v: dV formed) and the TMEM slot: in the
+  // alignment slack below the tiles when it has room, else after them (the
+  // request covers both)
   const bool low = sm - smem_raw >= 64;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(low ? smem_raw : sm + (SPLIT ? 11 : 7) * kTile);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 4);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(low ? smem_raw : sm + (SPLIT ? 9 : 7) * kTile);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 5);
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int bh = blockIdx.x, b = bh / p.heads, h = bh % p.heads;
@@ -288,6 +299,7 @@ __global__ void __launch_bounds__(kAttnThreads, SPLIT ? 1 : 2) attn_bwd_tc_k(con
     mbar_init(&bars[1], 1);
     mbar_init(&bars[2], kSoftmaxThreads);
     mbar_init(&bars[3], 1);
+    mbar_init(&bars[4], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&p.tm_qkv)) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&p.tm_do)) : "memory");
@@ -331,29 +343,38 @@ __global__ void __launch_bounds__(kAttnThreads, SPLIT ? 1 : 2) attn_bwd_tc_k(con
       tc_fence_after();
       constexpr uint32_t id_tt = instr_desc(64, true, true);    // dV, dK: A and B MN-major
       constexpr uint32_t id_nt = instr_desc(64, false, true);   // dQ: A K-major, B MN-major
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const uint32_t acc = k > 0 ? 1u : 0u;
-        // dV[j][d] = sum_i P[i][j] dO[i][d]
-        mma_f16(tmem + 128, smem_desc(smem_u32(sP) + 2048 * k, kTile, 1024),
-                smem_desc(smem_u32(sdO) + 2048 * k, kTile, 1024), id_tt, acc);
-        // dQ[i][d] = sum_j dS[i][j] K[j][d]
-        mma_f16(tmem, smem_desc(smem_u32(sdS) + (k >> 2) * kTile + 32 * (k & 3), 16, 1024),
+      // dV[j][d] = sum_i P[i][j] dO[i][d]
+      auto dv_mma = [&](int t, int k) {
+        mma_f16(tmem + 128, smem_desc(smem_u32(sP) + term_off(t) + 2048 * k, kTile, 1024),
+                smem_desc(smem_u32(sdO) + 2048 * k, kTile, 1024), id_tt, t + k > 0 ? 1u : 0u);
+      };
+      // dQ[i][d] = sum_j dS[i][j] K[j][d] and dK[j][d] = sum_i dS[i][j] Q[i][d]
+      auto dqk_mma = [&](int t, int k) {
+        const uint32_t ds = smem_u32(sdS) + term_off(t), acc = t + k > 0 ? 1u : 0u;
+        mma_f16(tmem, smem_desc(ds + (k >> 2) * kTile + 32 * (k & 3), 16, 1024),
                 smem_desc(smem_u32(sK) + 2048 * k, kTile, 1024), id_nt, acc);
-        // dK[j][d] = sum_i dS[i][j] Q[i][d]
-        mma_f16(tmem + 192, smem_desc(smem_u32(sdS) + 2048 * k, kTile, 1024),
-                smem_desc(smem_u32(sQ) + 2048 * k, kTile, 1024), id_tt, acc);
-      }
-      if constexpr (SPLIT)
+        mma_f16(tmem + 192, smem_desc(ds + 2048 * k, kTile, 1024), smem_desc(smem_u32(sQ) + 2048 * k, kTile, 1024),
+                id_tt, acc);
+      };
+      if constexpr (SPLIT) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {   // the same products of the remainders
-          mma_f16(tmem + 128, smem_desc(smem_u32(sPlo) + 2048 * k, kTile, 1024),
-                  smem_desc(smem_u32(sdO) + 2048 * k, kTile, 1024), id_tt, 1u);
-          mma_f16(tmem, smem_desc(smem_u32(sdSlo) + (k >> 2) * kTile + 32 * (k & 3), 16, 1024),
-                  smem_desc(smem_u32(sK) + 2048 * k, kTile, 1024), id_nt, 1u);
-          mma_f16(tmem + 192, smem_desc(smem_u32(sdSlo) + 2048 * k, kTile, 1024),
-                  smem_desc(smem_u32(sQ) + 2048 * k, kTile, 1024), id_tt, 1u);
+        for (int t = 0; t < kTerms; ++t)
+#pragma unroll
+          for (int k = 0; k < 8; ++k) dv_mma(t, k);
+        mma_commit(&bars[4]);
+        if (!mbar_wait(&bars[2], 1)) atomicExch(p.err, 16);   // dS in P's place
+        tc_fence_after();
+#pragma unroll
+        for (int t = 0; t < kTerms; ++t)
+#pragma unroll
+          for (int k = 0; k < 8; ++k) dqk_mma(t, k);
+      } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          dv_mma(0, k);
+          dqk_mma(0, k);
         }
+      }
       mma_commit(&bars[3]);
     }
   } else {
@@ -386,9 +407,10 @@ __global__ void __launch_bounds__(kAttnThreads, SPLIT ? 1 : 2) attn_bwd_tc_k(con
     if (!mbar_wait(&bars[1], 0)) atomicExch(p.err, 13);
     tc_fence_after();
     const uint32_t p_base = smem_u32(sP), ds_base = smem_u32(sdS);
-    const uint32_t pl_base = smem_u32(sPlo), dsl_base = smem_u32(sdSlo);
-#pragma unroll 1
-    for (int c = 2 * hf; c < 2 * hf + 2; ++c) {
+    // scores 32 cc .. +31 of this thread's 64: P into its tile, dS into its own
+    // or (SPLIT) `ds`
+    auto chunk = [&](int cc, float* ds) {
+      const int c = 2 * hf + cc;
       uint32_t rs[32], rp[32];
       tmem_ld32(trow + 32 * c, rs);
       tmem_ld32(trow + 128 + 32 * c, rp);
@@ -401,15 +423,36 @@ __global__ void __launch_bounds__(kAttnThreads, SPLIT ? 1 : 2) attn_bwd_tc_k(con
           const float pj = (live && j < n) ? attn_exp<SPLIT>(__uint_as_float(rs[8 * g + e]) * kScale - lse) : 0.f;
           pv[e] = pj;
           dv[e] = pj * (__uint_as_float(rp[8 * g + e]) - D) * kScale;
+          if (SPLIT) ds[32 * cc + 8 * g + e] = dv[e];
         }
         const uint32_t off = (c >> 1) * kTile + sw_off(i, (c & 1) * 4 + g);
-        st_unit<SPLIT>(p_base + off, pl_base + off, pv);
-        st_unit<SPLIT>(ds_base + off, dsl_base + off, dv);
+        st_unit<kTerms>(p_base + off, pv);
+        if (!SPLIT) st_unit<1>(ds_base + off, dv);
       }
+    };
+    auto release = [&] {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // P, dS visible to the tensor cores
+      tc_fence_before();
+      mbar_arrive(&bars[2]);
+    };
+    if constexpr (SPLIT) {
+      float ds[64];
+#pragma unroll
+      for (int cc = 0; cc < 2; ++cc) chunk(cc, ds);
+      release();
+      if (!mbar_wait(&bars[4], 0)) atomicExch(p.err, 17);   // P's tiles are free
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        float v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = ds[8 * u + e];
+        st_unit<kTerms>(ds_base + hf * kTile + sw_off(i, u), v);
+      }
+    } else {
+#pragma unroll 1
+      for (int cc = 0; cc < 2; ++cc) chunk(cc, nullptr);
     }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // P, dS visible to the tensor cores
-    tc_fence_before();
-    mbar_arrive(&bars[2]);
+    release();
     if (!mbar_wait(&bars[3], 0)) atomicExch(p.err, 14);
     tc_fence_after();
     // TMEM row i holds dQ row i and dK / dV row j = i; each half of the
@@ -433,22 +476,23 @@ __global__ void __launch_bounds__(kAttnThreads, SPLIT ? 1 : 2) attn_bwd_tc_k(con
 
 constexpr size_t kFwdSmem = 5 * kTile + 1024 + 64 + 4 * 128 * sizeof(float2);
 constexpr size_t kBwdSmem = 7 * kTile + 1024;   // 115,712 B: two CTAs in an SM's 228 KB
-constexpr size_t kBwdSplitSmem = 11 * kTile + 1024;
+constexpr size_t kFwdSplitSmem = 7 * kTile + 1024;   // two CTAs as well
+constexpr size_t kBwdSplitSmem = 9 * kTile + 1024;
 
 typedef void (*AttnKernel)(const AttnParams);
 struct AttnKernels {
   AttnKernel fwd, bwd;
-  size_t bwd_smem;
+  size_t fwd_smem, bwd_smem;
 };
 // The kernels of a head width, or nulls.
 AttnKernels attn_kernels(int dh) {
   switch (dh) {
-    case 16: return {attn_fwd_tc_k<16, true>, attn_bwd_tc_k<16, true>, kBwdSplitSmem};
-    case 32: return {attn_fwd_tc_k<32, true>, attn_bwd_tc_k<32, true>, kBwdSplitSmem};
-    case 48: return {attn_fwd_tc_k<48, true>, attn_bwd_tc_k<48, true>, kBwdSplitSmem};
-    case 64: return {attn_fwd_tc_k<64, false>, attn_bwd_tc_k<64, false>, kBwdSmem};
+    case 16: return {attn_fwd_tc_k<16, true>, attn_bwd_tc_k<16, true>, kFwdSplitSmem, kBwdSplitSmem};
+    case 32: return {attn_fwd_tc_k<32, true>, attn_bwd_tc_k<32, true>, kFwdSplitSmem, kBwdSplitSmem};
+    case 48: return {attn_fwd_tc_k<48, true>, attn_bwd_tc_k<48, true>, kFwdSplitSmem, kBwdSplitSmem};
+    case 64: return {attn_fwd_tc_k<64, false>, attn_bwd_tc_k<64, false>, kFwdSmem, kBwdSmem};
   }
-  return {nullptr, nullptr, 0};
+  return {nullptr, nullptr, 0, 0};
 }
 
 }  // namespace
@@ -485,7 +529,7 @@ AttnTcPlan* attention_tc_plan(const void* qkv, const void* out, const void* dout
   // which needs the largest shared-memory carveout (the default sizes the
   // carveout for one block).
   const int most = int(cudaSharedmemCarveoutMaxShared);
-  if (cudaFuncSetAttribute(a->k.fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kFwdSmem)) != cudaSuccess ||
+  if (cudaFuncSetAttribute(a->k.fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, int(a->k.fwd_smem)) != cudaSuccess ||
       cudaFuncSetAttribute(a->k.bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, int(a->k.bwd_smem)) != cudaSuccess ||
       cudaFuncSetAttribute(a->k.fwd, cudaFuncAttributePreferredSharedMemoryCarveout, most) != cudaSuccess ||
       cudaFuncSetAttribute(a->k.bwd, cudaFuncAttributePreferredSharedMemoryCarveout, most) != cudaSuccess) {
@@ -503,7 +547,7 @@ void attention_tc_fwd(const AttnTcPlan* a, const int32_t* len, void* out, float*
   p.out = static_cast<bf16*>(out);
   p.lse = lse;
   p.acc = 0;
-  launch_k(a->k.fwd, B * p.heads, kAttnThreads, kFwdSmem, st, p);
+  launch_k(a->k.fwd, B * p.heads, kAttnThreads, a->k.fwd_smem, st, p);
 }
 
 void attention_tc_bwd(const AttnTcPlan* a, const int32_t* len, const float* lse, void* dqkv, int B, bool acc,
