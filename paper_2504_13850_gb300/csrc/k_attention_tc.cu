@@ -106,6 +106,16 @@ __device__ __forceinline__ char* align1024(char* p) {
   return reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(p) + 1023) & ~uintptr_t(1023));
 }
 
+// Zeroes the DH columns of row r of a tile, half of them by each thread of the
+// row's pair.  A product with a zero P or dS would still be NaN where the other
+// operand's row is not finite: SPLIT clears the rows of masked keys and of the
+// next sequence, so that whatever those hold stays out, as on the CUDA cores.
+template <int DH>
+__device__ __forceinline__ void zero_row(const char* tile, int r, int hf) {
+#pragma unroll
+  for (int u = 0; u < DH / 16; ++u) st_shared4(smem_u32(tile) + sw_off(r, hf * (DH / 16) + u), 0u, 0u, 0u, 0u);
+}
+
 // The first N accumulator columns of this lane's row -> N bf16 at dst
 // (optionally added to what is there).
 template <int N>
@@ -240,6 +250,7 @@ __global__ void __launch_bounds__(kAttnThreads, 1) attn_fwd_tc_k(const __grid_co
         st_unit<kTerms>(p_base + sw_off(i, c * 4 + g), v);
       }
     }
+    if (SPLIT && i >= n) zero_row<DH>(sV, i, hf);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // P~ visible to the tensor cores
     tc_fence_before();
     mbar_arrive(&bars[2]);
@@ -420,9 +431,11 @@ __global__ void __launch_bounds__(kAttnThreads, SPLIT ? 1 : 2) attn_bwd_tc_k(con
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           const int j = 32 * c + 8 * g + e;
-          const float pj = (live && j < n) ? attn_exp<SPLIT>(__uint_as_float(rs[8 * g + e]) * kScale - lse) : 0.f;
+          const bool in = live && j < n;
+          const float pj = in ? attn_exp<SPLIT>(__uint_as_float(rs[8 * g + e]) * kScale - lse) : 0.f;
           pv[e] = pj;
           dv[e] = pj * (__uint_as_float(rp[8 * g + e]) - D) * kScale;
+          if (SPLIT && !in) dv[e] = 0.f;
           if (SPLIT) ds[32 * cc + 8 * g + e] = dv[e];
         }
         const uint32_t off = (c >> 1) * kTile + sw_off(i, (c & 1) * 4 + g);
@@ -439,6 +452,11 @@ __global__ void __launch_bounds__(kAttnThreads, SPLIT ? 1 : 2) attn_bwd_tc_k(con
       float ds[64];
 #pragma unroll
       for (int cc = 0; cc < 2; ++cc) chunk(cc, ds);
+      if (i >= n) zero_row<DH>(sK, i, hf);
+      if (!live) {
+        zero_row<DH>(sQ, i, hf);
+        zero_row<DH>(sdO, i, hf);
+      }
       release();
       if (!mbar_wait(&bars[4], 0)) atomicExch(p.err, 17);   // P's tiles are free
 #pragma unroll
@@ -463,6 +481,9 @@ __global__ void __launch_bounds__(kAttnThreads, SPLIT ? 1 : 2) attn_bwd_tc_k(con
       const uint32_t col = t == 0 ? 0u : (t == 1 ? 192u : 128u);     // dQ, dK, dV
       uint32_t r[32];
       tmem_ld32(trow + col + DH / 2 * hf, r);
+      if (SPLIT && t > 0 && i >= n)
+#pragma unroll
+        for (int e = 0; e < 32; ++e) r[e] = 0u;   // no gradient of a masked key
       if (live) store_row<DH / 2>(drow + t * p.C + h * DH + DH / 2 * hf, r, p.acc != 0);
     }
   }

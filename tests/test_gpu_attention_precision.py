@@ -35,9 +35,8 @@ class DeviceArray:
         self.__cuda_array_interface__ = {"shape": shape, "typestr": typestr, "data": (ptr, False), "version": 3}
 
 
-def attention_step(width, heads, L, B, seed, poke=None):
-    """Runs one step; returns ({name: bf16 values of the step}, {name: exact}) of O, dQ, dK, dV, [B, heads, L, width].
-    `poke(q, k, v, lens)` may change the projections and the lengths in place before the step."""
+def attention_step(width, heads, L, B, seed):
+    """Runs one step; returns ({name: bf16 values of the step}, {name: exact}) of O, dQ, dK, dV, [B, heads, L, width]."""
     C, D = width * heads, (B * L + 63) // 64 * 64
     ops = [dict(kind="linear", in0=0, cin=D, cout=3 * C, bias=0), dict(kind="attention", in0=1, c=C, heads=heads),
            dict(kind="flatten", in0=2), dict(kind="linear", in0=3, cin=L * C, cout=CLASSES, bias=0)]
@@ -49,9 +48,6 @@ def attention_step(width, heads, L, B, seed, poke=None):
     head[0] = sign * 2.0 ** -torch.randint(6, 10, (L * C,), generator=g, device="cuda")
     lens = torch.randint(max(1, L // 4), L + 1, (B,), generator=g, device="cuda", dtype=torch.int32)
     labels = torch.randint(0, CLASSES, (B,), generator=g, device="cuda", dtype=torch.int32)
-    if poke:
-        poke(*qkv, lens)
-        w[:, :B * L] = qkv.permute(1, 3, 0, 2, 4).reshape(B * L, 3 * C).t()
     x = torch.zeros(B * L, D, device="cuda", dtype=torch.bfloat16)
     x[torch.arange(B * L), torch.arange(B * L)] = 1
     x = x.reshape(B, L, 1, D)
@@ -70,8 +66,6 @@ def attention_step(width, heads, L, B, seed, poke=None):
     s.close()
     q, k, v = qkv.double()
     dead = torch.arange(L, device="cuda") >= lens.view(B, 1, 1)
-    for t in (k, v):      # masked keys take no part, whatever they hold
-        t.masked_fill_(dead.view(B, 1, L, 1), 0.0)
     score = (q @ k.transpose(-1, -2) / math.sqrt(width)).masked_fill(dead.view(B, 1, 1, L), -math.inf)
     p = score.softmax(-1)
     dz = (logits.softmax(-1) - torch.nn.functional.one_hot(labels.long(), CLASSES)) / B
@@ -90,3 +84,44 @@ def test_fp32_probabilities(width, heads, L, B):
         for n in got:
             off.setdefault(n, []).append((got[n] != exact[n].float().bfloat16().double()).double().mean().item())
     assert all(sum(v) / len(v) <= 2.0 ** -10 for v in off.values()), off
+
+
+@pytest.mark.parametrize("width,heads,L", [(16, 2, 9), (32, 4, 77), (48, 2, 127), (24, 4, 100)])
+@pytest.mark.parametrize("value", [math.inf, math.nan])
+def test_masked_keys_and_other_sequences_stay_out(width, heads, L, value):
+    """Keys past a sequence's length that hold infinities or NaN, and a whole
+    sequence of them, change nothing of the other sequences.  The packed q|k|v
+    passes a unit affine, whose shift gradient is the column sum of d(q|k|v)."""
+    B, C = 4, width * heads
+    ops = [dict(kind="affine", in0=0, c=3 * C), dict(kind="attention", in0=1, c=C, heads=heads),
+           dict(kind="flatten", in0=2), dict(kind="linear", in0=3, cin=L * C, cout=CLASSES, bias=0)]
+    g = torch.Generator(device="cuda").manual_seed(7)
+    x = torch.randn(B, L, 1, 3 * C, generator=g, device="cuda").bfloat16()
+    head = torch.randn(CLASSES, L * C, generator=g, device="cuda") * math.sqrt(2.0 / (L * C))
+    lens = torch.randint(max(1, L // 4), L, (B,), generator=g, device="cuda", dtype=torch.int32)   # one masked key at least
+    labels = torch.arange(B, device="cuda", dtype=torch.int32)
+    theta = torch.cat([torch.ones(3 * C, device="cuda"), torch.zeros(3 * C, device="cuda"), head.flatten()]).cpu().numpy()
+
+    def step(batch):
+        s = api.Server(ops, 1, 1, 1, B, (L, 1, 3 * C), CLASSES, "bf16", 0.0, 0.0, seq=True)
+        s.set_params(theta)
+        torch.cuda.synchronize()
+        assert s.enqueue_activations(0, batch, labels, lens)[0] == api.OK
+        s.server_step()
+        s.synchronize()
+        s.check_error()
+        o = torch.as_tensor(DeviceArray(s.tensor(2)[0], (B, L, C), "<i2"), device="cuda").view(torch.bfloat16).clone()
+        v = s.get_momentum()
+        s.close()
+        return o, v[3 * C:6 * C]
+
+    o0, shift0 = step(x)
+    y = x.clone()
+    for b in range(B):
+        y[b, lens[b]:, :, C:] = value       # keys and values only: every query still counts
+    o1, shift1 = step(y)
+    assert torch.equal(o1, o0) and (shift1 == shift0).all()
+    y[1] = value
+    o2, _ = step(y)
+    keep = [0, 2, 3]
+    assert torch.equal(o2[keep], o0[keep])
