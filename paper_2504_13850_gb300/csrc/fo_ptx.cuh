@@ -54,6 +54,18 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
     if (global_ns() - t0 > 2000000000ull) return false;
   }
 }
+// The same for a warp whose lanes go on together: each lane has its own clock,
+// so that near the limit some may see the phase complete and others give up,
+// and instructions for the whole warp behind such a wait would hang.  Every
+// wait ends, so the vote does, and all lanes get its answer.  (A loop that one
+// lane can run by itself does so inside `if (elect_one())` with mbar_wait.)
+__device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity));
+}
+// True in all lanes of a warp if any of them sees the flag.
+__device__ __forceinline__ bool warp_flag(const volatile int* flag) {
+  return __any_sync(0xffffffffu, *flag != 0);
+}
 __device__ __forceinline__ void tma_2d(void* dst, const CUtensorMap* m, uint64_t* bar, int c0, int c1) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"

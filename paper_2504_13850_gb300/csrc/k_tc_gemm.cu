@@ -255,8 +255,8 @@ int active_clusters(TcContext* c, int kind, int bn, int S, int epi) {
 
 // Tile width and K split from a cost model in microseconds,
 // fitted to GB300 timelines of these kernels:
-//  * a k-block stage alone costs 0.204 / 0.231 / 0.345 us at widths 64 / 128
-//    / 256 (32 k-blocks a tile, every SM busy; MN-major 0.258 / 0.398 at 128 /
+//  * a k-block stage alone costs 0.165 / 0.212 / 0.332 us at widths 64 / 128
+//    / 256 (32 k-blocks a tile, every SM busy; MN-major 0.250 / 0.390 at 128 /
 //    256): narrow tiles are bounded by the round of mbarrier waits and the MMA
 //    issue of a stage, the 256-wide tile by 192 KB in flight over a TMA round
 //    trip of ~1.4 us.  In a step, narrow tiles cost the kernels beside them

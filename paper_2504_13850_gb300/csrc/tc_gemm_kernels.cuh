@@ -384,13 +384,14 @@ struct KindTraits {
 
 // The MMAs of one pipeline stage (operands A then B at shared address `a0`)
 // into the accumulator at `d`, added to it when `acc`, and their commit to
-// `empty`.  Called by the one lane that elect_one picked in a converged warp:
-// the compiler then knows that descriptors and addresses are uniform.  In a
-// branch on the lane number it moved each of them through a per-lane path,
-// which cost ~0.08 us a stage and bounded every tile narrower than 256 (32
-// k-blocks a tile, 152 CTAs: 0.283 -> 0.204 us a stage at BN = 64, 0.288 ->
-// 0.231 at 128 K-major, 0.292 -> 0.258 MN-major; 256 is bounded by its bytes
-// in flight, 0.345).
+// `empty`.  Called by the one lane that elect_one picked in a converged warp,
+// which runs the whole loop, waits included: the compiler then knows that
+// descriptors and addresses are uniform, and no lane's view of a wait that ran
+// out can part it from others it would meet again.  us a stage (32 k-blocks a
+// tile, 152 CTAs; in a branch on the lane number / with all lanes waiting and
+// one elected for each stage / here): 0.283 / 0.204 / 0.165 at BN = 64, 0.288 /
+// 0.230 / 0.212 at 128 K-major, 0.292 / 0.255 / 0.250 MN-major; 256 is bounded
+// by its bytes in flight, 0.340 / 0.332 for the last two.
 template <int KIND, int BN>
 __device__ __forceinline__ void mma_stage(uint32_t d, uint32_t a0, bool acc, uint64_t* empty) {
   constexpr bool amn = KindTraits<KIND>::a_mn, bmn = KindTraits<KIND>::b_mn;
@@ -599,36 +600,36 @@ __global__ void __launch_bounds__(kThreads, 1) tc_gemm_kernel(const __grid_const
   pdl_wait();      // the previous kernel's writes are visible from here on
 
   if (warp == 0) {
-    KLoader<KIND, BN, EPI> ld;
-    ld.init(p, m0, n0, kb0);
-    for (int it = 0; it < nk; ++it, ld.next(p)) {
-      const int s = it % STAGES;
-      if (!mbar_wait(&empty[s], ((it / STAGES) & 1) ^ 1)) {
-        atomicExch(p.err, 1);
-        *abort_flag = 1;
-        break;
-      }
-      if (*abort_flag) break;
-      if (elect_one()) {
+    if (elect_one()) {
+      KLoader<KIND, BN, EPI> ld;
+      ld.init(p, m0, n0, kb0);
+      for (int it = 0; it < nk; ++it, ld.next(p)) {
+        const int s = it % STAGES;
+        if (!mbar_wait(&empty[s], ((it / STAGES) & 1) ^ 1)) {
+          atomicExch(p.err, 1);
+          *abort_flag = 1;
+          break;
+        }
+        if (*abort_flag) break;
         char* sa = smem + s * STAGE_BYTES;
         mbar_expect_tx(&full[s], STAGE_BYTES);
         ld.load(p, sa, sa + A_BYTES, &full[s]);
       }
     }
   } else if (warp == 1) {
-    bool ok = true;
-    for (int it = 0; it < nk; ++it) {
-      const int s = it % STAGES;
-      if (!mbar_wait(&full[s], (it / STAGES) & 1)) {
-        atomicExch(p.err, 2);
-        *abort_flag = 1;
-        ok = false;
-        break;
-      }
-      tc_fence_after();
-      if (elect_one()) mma_stage<KIND, BN>(tmem, smem_u32(smem + s * STAGE_BYTES), it > 0, &empty[s]);
-    }
     if (elect_one()) {
+      bool ok = true;
+      for (int it = 0; it < nk; ++it) {
+        const int s = it % STAGES;
+        if (!mbar_wait(&full[s], (it / STAGES) & 1)) {
+          atomicExch(p.err, 2);
+          *abort_flag = 1;
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        mma_stage<KIND, BN>(tmem, smem_u32(smem + s * STAGE_BYTES), it > 0, &empty[s]);
+      }
       if (ok) mma_commit(accum);
       else mbar_expect_tx(accum, 0);  // release the epilogue without data
     }
@@ -906,18 +907,18 @@ __global__ void __launch_bounds__(kPersistThreads, 1) tc_gemm_persistent(const _
   pdl_wait();
 
   if (warp == 0) {
-    uint32_t g = 0;
-    for (int t = unit; t < tiles && !*abort_flag; t += units) {
-      KLoader<KIND, BN, EPI> ld;
-      ld.init(p, tile_m0(t), tile_n0(t), 0);
-      for (int kb = 0; kb < KB; ++kb, ++g, ld.next(p)) {
-        const int s = g % STAGES;
-        if (!mbar_wait(&empty[s], ((g / STAGES) & 1) ^ 1)) {
-          atomicExch(p.err, 4);
-          *abort_flag = 1;
-          break;
-        }
-        if (elect_one()) {
+    if (elect_one()) {
+      uint32_t g = 0;
+      for (int t = unit; t < tiles && !*abort_flag; t += units) {
+        KLoader<KIND, BN, EPI> ld;
+        ld.init(p, tile_m0(t), tile_n0(t), 0);
+        for (int kb = 0; kb < KB; ++kb, ++g, ld.next(p)) {
+          const int s = g % STAGES;
+          if (!mbar_wait(&empty[s], ((g / STAGES) & 1) ^ 1)) {
+            atomicExch(p.err, 4);
+            *abort_flag = 1;
+            break;
+          }
           char* sa = smem + s * STAGE_BYTES;
           mbar_expect_tx(&full[s], STAGE_BYTES);
           ld.load(p, sa, sa + A_BYTES, &full[s]);
@@ -925,37 +926,38 @@ __global__ void __launch_bounds__(kPersistThreads, 1) tc_gemm_persistent(const _
       }
     }
   } else if (warp == 1) {
-    uint32_t g = 0, lt = 0;
-    for (int t = unit; t < tiles && !*abort_flag; t += units, ++lt) {
-      const uint32_t b = lt & 1;
-      // E_TMA: the epilogue warps arrive once per buffer before the first
-      // tile, after writing its starting value
-      if (!mbar_wait(&acc_empty[b], ((lt >> 1) & 1) ^ ((EPI & E_TMA) ? 0u : 1u))) {
-        atomicExch(p.err, 5);
-        *abort_flag = 1;
-        if (elect_one()) mbar_expect_tx(&acc_full[b], 0);
-        break;
-      }
-      tc_fence_after();
-      const uint32_t d = tmem + b * BN;
-      bool ok = true;
-      for (int kb = 0; kb < KB; ++kb, ++g) {
-        const int s = g % STAGES;
-        if (!mbar_wait(&full[s], (g / STAGES) & 1)) {
-          atomicExch(p.err, 6);
+    if (elect_one()) {
+      uint32_t g = 0, lt = 0;
+      for (int t = unit; t < tiles && !*abort_flag; t += units, ++lt) {
+        const uint32_t b = lt & 1;
+        // E_TMA: the epilogue warps arrive once per buffer before the first
+        // tile, after writing its starting value
+        if (!mbar_wait(&acc_empty[b], ((lt >> 1) & 1) ^ ((EPI & E_TMA) ? 0u : 1u))) {
+          atomicExch(p.err, 5);
           *abort_flag = 1;
-          ok = false;
+          mbar_expect_tx(&acc_full[b], 0);
           break;
         }
         tc_fence_after();
-        if (elect_one())
+        const uint32_t d = tmem + b * BN;
+        bool ok = true;
+        for (int kb = 0; kb < KB; ++kb, ++g) {
+          const int s = g % STAGES;
+          if (!mbar_wait(&full[s], (g / STAGES) & 1)) {
+            atomicExch(p.err, 6);
+            *abort_flag = 1;
+            ok = false;
+            break;
+          }
+          tc_fence_after();
           mma_stage<KIND, BN>(d, smem_u32(smem + s * STAGE_BYTES), (EPI & E_TMA) || kb > 0, &empty[s]);
-      }
-      if (elect_one()) {
+        }
         if (ok) mma_commit(&acc_full[b]);
-        else mbar_expect_tx(&acc_full[b], 0);
+        else {
+          mbar_expect_tx(&acc_full[b], 0);
+          break;
+        }
       }
-      if (!ok) break;
     }
   } else if constexpr ((EPI & E_TMA) != 0) {
     // Epilogue through TMA stores: warp w (2..9) owns TMEM lanes
@@ -978,13 +980,13 @@ __global__ void __launch_bounds__(kPersistThreads, 1) tc_gemm_persistent(const _
     for (int t = unit; t < tiles; t += units, ++lt) {
       const uint32_t b = lt & 1;
       const int n0 = tile_n0(t) + half * CW, m0 = tile_m0(t) + q * 32;
-      const bool ready = mbar_wait(&acc_full[b], (lt >> 1) & 1);
+      const bool ready = warp_wait(&acc_full[b], (lt >> 1) & 1);
       tc_fence_after();
       if (!ready) {
         atomicExch(p.err, 7);
         *abort_flag = 1;
       }
-      if (!ready || *abort_flag) break;
+      if (!ready || warp_flag(abort_flag)) break;
       const uint32_t trow = tq + b * BN;
       uint32_t cur[32], nxt[32];
       tmem_ld32_issue(trow, cur);
@@ -1053,13 +1055,13 @@ __global__ void __launch_bounds__(kPersistThreads, 1) tc_gemm_persistent(const _
       const int n0 = tile_n0(t), m0 = tile_m0(t);
       float bnext[8];
       load_bias8<EPI>(p, lane, n0 + half * CW, bnext);   // in flight during the wait
-      const bool ready = mbar_wait(&acc_full[b], (lt >> 1) & 1);
+      const bool ready = warp_wait(&acc_full[b], (lt >> 1) & 1);
       tc_fence_after();
       if (!ready) {
         atomicExch(p.err, 7);
         *abort_flag = 1;
       }
-      if (!ready || *abort_flag) break;
+      if (!ready || warp_flag(abort_flag)) break;
       const uint32_t stage = smem_u32(stage_all) + uint32_t(warp - 2) * 4096u;
       const uint32_t trow = tmem + b * BN + (uint32_t(q * 32) << 16);
       // Software-pipelined: the TMEM load of chunk c + 32 is in flight while
