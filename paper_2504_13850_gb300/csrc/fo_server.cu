@@ -10,6 +10,7 @@
 
 #include <memory>
 #include "fo_tc.h"
+#include "fo_upload.hpp"
 
 #include <array>
 #include <cstring>
@@ -1402,6 +1403,10 @@ static int server_create(const fo_op* ops, int n_ops, const fo_optimizer* opt, c
   }
   s->sched = new fo::TaskScheduler(c.num_devices, c.omega, c.depth, c.sched_policy);
   s->use_side = getenv("FO_NO_SIDE") == nullptr;
+  if (cudaGetDevice(&s->device) != cudaSuccess) {
+    destroy_impl(s);
+    return set_err(FO_ERR_CUDA, "no current device");
+  }
   if (cudaStreamCreateWithFlags(&s->cs, cudaStreamNonBlocking) != cudaSuccess ||
       cudaStreamCreateWithFlags(&s->xs, cudaStreamNonBlocking) != cudaSuccess ||
       cudaStreamCreateWithFlags(&s->hs, cudaStreamNonBlocking) != cudaSuccess ||
@@ -1502,15 +1507,31 @@ int fo_server_store_params_device(fo_server* s, float* dst, int64_t n) {
   return FO_OK;
 }
 
-// True for memory of the current device at a multiple of `align` bytes, which a kernel may read.
-static bool on_device(const void* p, uintptr_t align) {
+// True if the upload kernel may read `bytes` bytes at p (fo_upload.hpp).
+static bool kernel_may_read(const fo_server* s, const void* p, size_t bytes, size_t align) {
+  typedef CUresult (*AddressRange)(CUdeviceptr*, size_t*, CUdeviceptr);
+  static const AddressRange range = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+        q != cudaDriverEntryPointSuccess)
+      f = nullptr;
+    return reinterpret_cast<AddressRange>(f);
+  }();
   cudaPointerAttributes a{};
   int dev = -1;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  return a.type == cudaMemoryTypeDevice && a.device == dev && reinterpret_cast<uintptr_t>(p) % align == 0;
+  fo::MemoryRange m{a.type == cudaMemoryTypeDevice, a.device, 0, 0};
+  CUdeviceptr base = 0;
+  size_t length = 0;
+  if (m.device && range && range(&base, &length, reinterpret_cast<CUdeviceptr>(p)) == CUDA_SUCCESS) {
+    m.base = uintptr_t(base);
+    m.length = length;
+  }
+  return fo::upload_kernel_may_read(m, reinterpret_cast<uintptr_t>(p), bytes, align, s->device, dev);
 }
 
 // The copies of an accepted upload into batch slot `slot` (before the
@@ -1527,7 +1548,8 @@ static int upload_copies(fo_server* s, int32_t slot, const void* acts, const int
     if (q == cudaErrorNotReady) busy = true;
     else FO_CUDA(q);
   }
-  if (!busy && on_device(acts, 16) && on_device(labels, 4) && (!lengths || on_device(lengths, 4))) {
+  if (!busy && kernel_may_read(s, acts, size_t(s->slot_act_bytes), 16) && kernel_may_read(s, labels, size_t(B) * 4, 4) &&
+      (!lengths || kernel_may_read(s, lengths, size_t(B) * 4, 4))) {
     fo::upload_copy(acts, d_act, s->slot_act_bytes, labels, d_lab, lengths, d_len, B, s->hs);
     FO_CUDA(cudaGetLastError());
     FO_CUDA(cudaEventRecord(s->slot_ready[slot], s->hs));

@@ -128,6 +128,7 @@ struct fo_server {
   float* row_loss = nullptr;
   int64_t* d_step = nullptr;   // device copy of steps_done (indexes the loss ring)
   bool use_graphs = true;
+  int device = -1;             // the CUDA device the server was created on
   std::vector<cudaGraphExec_t> graphs, prof_graphs;  // per batch slot
   std::vector<std::vector<struct ProfRec>> prof_events;
   int64_t steps_done = 0;
