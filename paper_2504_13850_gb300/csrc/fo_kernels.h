@@ -201,9 +201,9 @@ void layernorm_bwd8_pass(const void* x, const float* gamma, const float* mean, c
 
 
 // One upload from device memory: `bytes` of activations (src 16-byte aligned)
-// and B labels and, when given, lengths.
-void upload_copy(const void* acts, void* d_acts, int64_t bytes, const int32_t* labels, int32_t* d_labels,
-                 const int32_t* lengths, int32_t* d_lengths, int B, cudaStream_t st);
+// and B labels and, when given, lengths.  Returns the launch's own status.
+cudaError_t upload_copy(const void* acts, void* d_acts, int64_t bytes, const int32_t* labels, int32_t* d_labels,
+                        const int32_t* lengths, int32_t* d_lengths, int B, cudaStream_t st);
 
 // ---- MobileNetV3 bottleneck (k_mobile.cu) ----
 // Depthwise k x k convolution, NHWC, weights [C][k][k] in the activation

@@ -32,8 +32,10 @@ int set_err(int code, const std::string& msg) {
 #define FO_CUDA(call)                                                                   \
   do {                                                                                  \
     cudaError_t e_ = (call);                                                            \
-    if (e_ != cudaSuccess)                                                              \
+    if (e_ != cudaSuccess) {                                                            \
+      cudaGetLastError(); /* reported here: not again by a later call's check */        \
       return set_err(FO_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
+    }                                                                                   \
   } while (0)
 
 }  // namespace
@@ -1550,8 +1552,7 @@ static int upload_copies(fo_server* s, int32_t slot, const void* acts, const int
   }
   if (!busy && kernel_may_read(s, acts, size_t(s->slot_act_bytes), 16) && kernel_may_read(s, labels, size_t(B) * 4, 4) &&
       (!lengths || kernel_may_read(s, lengths, size_t(B) * 4, 4))) {
-    fo::upload_copy(acts, d_act, s->slot_act_bytes, labels, d_lab, lengths, d_len, B, s->hs);
-    FO_CUDA(cudaGetLastError());
+    FO_CUDA(fo::upload_copy(acts, d_act, s->slot_act_bytes, labels, d_lab, lengths, d_len, B, s->hs));
     FO_CUDA(cudaEventRecord(s->slot_ready[slot], s->hs));
     FO_CUDA(cudaEventSynchronize(s->slot_ready[slot]));   // the caller may reuse its buffers
     return FO_OK;

@@ -381,14 +381,18 @@ __global__ void __launch_bounds__(256) upload_copy_k(const uint4* __restrict__ a
   }
   for (; i < n16; i += step) da[i] = a[i];
 }
-void upload_copy(const void* acts, void* d_acts, int64_t bytes, const int32_t* labels, int32_t* d_labels,
-                 const int32_t* lengths, int32_t* d_lengths, int B, cudaStream_t st) {
+cudaError_t upload_copy(const void* acts, void* d_acts, int64_t bytes, const int32_t* labels, int32_t* d_labels,
+                        const int32_t* lengths, int32_t* d_lengths, int B, cudaStream_t st) {
   const int64_t n16 = bytes / 16;
   const int nt = int(bytes % 16);
   // at least one thread per label (B <= 1024) and tail byte
   const int blocks = elementwise_blocks(std::max<int64_t>(n16 / 4, std::max(B, 16)), 256);
-  upload_copy_k<<<blocks, 256, 0, st>>>((const uint4*)acts, (uint4*)d_acts, n16, (const char*)acts + 16 * n16,
-                                        (char*)d_acts + 16 * n16, nt, labels, d_labels, lengths, d_lengths, B);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(unsigned(blocks));
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  return cudaLaunchKernelEx(&cfg, upload_copy_k, (const uint4*)acts, (uint4*)d_acts, n16, (const char*)acts + 16 * n16,
+                            (char*)d_acts + 16 * n16, nt, labels, d_labels, lengths, d_lengths, B);
 }
 
 // -------------------------------------------------------------- avgpool

@@ -1,6 +1,6 @@
 """Which uploads the copy kernel takes, and what becomes of the others: the host
 rule over device, extent and alignment (CPU), and buffers that end before the
-batch does, which get an error (GPU)."""
+batch does, which get an error and leave the server usable (GPU)."""
 import ctypes as C
 import os
 import shutil
@@ -71,6 +71,9 @@ def test_buffer_that_ends_early_is_refused(short):
         args[0 if short == "acts" else 1] = tail
         rc = api.lib().fo_enqueue_activations(s.h, 0, *args, None, C.byref(on))
         assert rc == api.ERR_CUDA
+        assert s.enqueue_activations(0, acts, labels)[0] == api.OK          # the server goes on
+        assert s.server_step()[0] == api.OK
+        assert np.isfinite(s.read_losses(0, 1)).all()
     finally:
         s.close()
         rt.cudaFree(ptr)
