@@ -277,6 +277,15 @@ __global__ void head_wgrad_k(const float* __restrict__ dz, const T* __restrict__
   }
 }
 
+// Floats of the head's shared memory: logits of R rows, this CTA's share of
+// them, and the partial sums of both products: of the logits R x per x (8 /
+// warps over class groups), at most R x max(per, 32), and of dx R x 256 V.
+size_t head_floats(int R, int V, int C) {
+  const int per = (C + kHeadCtas - 1) / kHeadCtas;
+  return size_t(R) * (size_t(C) + per + std::max(kHeadThreads * V, std::max(per, 32)));
+}
+constexpr int kHeadMaxClasses = 1024;   // more classes take the unfused loss
+
 }  // namespace
 
 void head_forward_loss(const void* x, int dt, const float* W, const float* bias, const int32_t* labels, int B,
@@ -286,13 +295,12 @@ void head_forward_loss(const void* x, int dt, const float* W, const float* bias,
   int R = 1;
   while (R < 8 && (B + R - 1) / R > 16) R *= 2;
   const int V = K % 4 == 0 ? 4 : 1;   // rows of W and x stay aligned
-  const int per = (C + kHeadCtas - 1) / kHeadCtas;
-  // partials of the logits: R x per x (8 / warps over class groups), at most R x max(per, 32); of dx: R x 256 V
-  const size_t part = std::max<size_t>(size_t(kHeadThreads) * V, std::max(per, 32));
-  const size_t sm = sizeof(float) * R * (size_t(C) + per + part);
+  const size_t sm = sizeof(float) * head_floats(R, V, C);
   auto go = [&](auto kernel, auto tag) {
     typedef decltype(tag) T;
-    if (sm > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(sm));
+    // the same limit in every call: servers of other class counts may launch from other threads meanwhile
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         int(sizeof(float) * head_floats(R, V, kHeadMaxClasses)));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(unsigned((B + R - 1) / R) * kHeadCtas);
     cfg.blockDim = dim3(kHeadThreads);
