@@ -160,8 +160,11 @@ FO_API int fo_server_get_momentum(fo_server* s, float* host, int64_t n);
  *   the last fo_server_step.  The pointer stays valid for the server's
  *   lifetime; the contents change with each step, which runs on
  *   fo_server_stream.  A flatten of the uploaded batch is a view of it: its
- *   pointer is the batch slot the last step read.  FO_ERR_ARG for an index
- *   outside 1..n_ops.
+ *   pointer is the batch slot the last step read.  Outputs that the step never
+ *   forms on their own are not written: what a ReLU behind a convolution,
+ *   linear layer, affine or add reads, what a max-pool in a convolution's
+ *   epilogue reads, and a residual add's operand that a GEMM adds to the other
+ *   one as it stores it.  FO_ERR_ARG for an index outside 1..n_ops.
  * fo_server_params_device: the fp32 master parameters on the device in the
  *   server's padded layout (*n floats; identical for servers built from the
  *   same op list), for device-to-device aggregation.  Read it only when the

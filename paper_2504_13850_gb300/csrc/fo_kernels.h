@@ -171,9 +171,9 @@ void finish_batched(const std::vector<FinishTask>& tasks, cudaStream_t st);
 int affine_bwd8_chunks(int64_t rows, int C);
 void affine_bwd8_pass(const void* dy, const void* x, const float* scale, void* dx, bool acc, int64_t rows, int C,
                       float* p_scale, float* p_shift, cudaStream_t st, const void* hswish_in = nullptr);
-// y = [relu](bf16(x * sc + sh) + r), r = x2 or (sc2 given) bf16(x2 * sc2 + sh2).
+// f = bf16(x * sc + sh), y = [relu](f + r), r = x2 or (sc2 given) f2 = bf16(x2 * sc2 + sh2).
 void affine_add_x8(const void* x, const float* sc, const float* sh, const void* x2, const float* sc2,
-                   const float* sh2, void* y, int64_t n, int C, bool relu, cudaStream_t st);
+                   const float* sh2, void* f, void* f2, void* y, int64_t n, int C, bool relu, cudaStream_t st);
 // Affine then hard swish in one pass: pre = x * scale + shift, post = hswish(pre).
 void affine_hswish_fwd_x8(const void* x, const float* sc, const float* sh, void* pre, void* post, int64_t n, int C,
                           cudaStream_t st);

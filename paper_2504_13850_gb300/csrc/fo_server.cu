@@ -227,7 +227,7 @@ struct Fusion {
   // the GELU too (the plan decides; the GELU op runs alone otherwise).
   std::vector<int> gelu_of;    // producer op -> the GELU op, or -1
   // Residual add whose operand is an affine's output that nothing else reads:
-  // the add forms it on the fly (its backward needs only the add's mask).
+  // the add forms (and stores) it.
   std::vector<std::array<int, 2>> add_affine;   // add op -> per operand (in0, in1): the affine op, or -1
   bool head = false;           // last linear + loss handled by the head kernels
 };
@@ -495,9 +495,10 @@ int build_plan(fo_server* s) {
           const int pa = p0 >= 0 ? p0 : p1;                    // the first operand's affine
           const int pb = p0 >= 0 ? p1 : -1;                    // the second's, if it has one
           const int xa = s->ops[pa].in0, xb = pb >= 0 ? s->ops[pb].in0 : (p0 >= 0 ? b : a);
-          add("affine_add_fwd", 1, 0.0, 3 * tbytes(i + 1), [=](cudaStream_t st) {
+          add("affine_add_fwd", 1, 0.0, (pb >= 0 ? 5 : 4) * tbytes(i + 1), [=](cudaStream_t st) {
             fo::affine_add_x8(act(xa), P(s, pa, 0), P(s, pa, 1), act(xb), pb >= 0 ? P(s, pb, 0) : nullptr,
-                              pb >= 0 ? P(s, pb, 1) : nullptr, s->T[o].act, s->T[o].numel(), s->T[o].C, relu, st);
+                              pb >= 0 ? P(s, pb, 1) : nullptr, s->T[pa + 1].act, pb >= 0 ? s->T[pb + 1].act : nullptr,
+                              s->T[o].act, s->T[o].numel(), s->T[o].C, relu, st);
           });
           break;
         }

@@ -155,12 +155,13 @@ __global__ void __launch_bounds__(256) affine_fwd_x8_k(const bf16* __restrict__ 
 
 // A residual add (and the ReLU after it) of an affine's output and a second
 // operand, itself an affine's output when sc2 is given: y = affine(x) +
-// [affine2](x2), with the affine outputs rounded to bf16 as their own pass
-// would store them.
+// [affine2](x2), with the affine outputs rounded to bf16 and stored (to f, f2)
+// as by their own pass.
 template <bool TWO>
 __global__ void __launch_bounds__(256) affine_add_x8_k(const bf16* __restrict__ x, const float* __restrict__ sc,
                                                        const float* __restrict__ sh, const bf16* __restrict__ x2,
                                                        const float* __restrict__ sc2, const float* __restrict__ sh2,
+                                                       bf16* __restrict__ f, bf16* __restrict__ f2,
                                                        bf16* __restrict__ y, int64_t n8, int C, int relu) {
   pdl_wait();
   pdl_trigger();
@@ -171,7 +172,11 @@ __global__ void __launch_bounds__(256) affine_add_x8_k(const bf16* __restrict__ 
   GRID_STRIDE8(i, n8) {
     const V8 p = ld8(x + 8 * i), r = ld8(x2 + 8 * i);
     V8 o = af(p), q = r;
-    if (TWO) q = ag(r);
+    st8(f + 8 * i, o);
+    if (TWO) {
+      q = ag(r);
+      st8(f2 + 8 * i, q);
+    }
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
       const float v = round_bf16(o.v[j]) + (TWO ? round_bf16(q.v[j]) : q.v[j]);
@@ -779,9 +784,9 @@ void affine_fwd_x8(const void* x, const float* sc, const float* sh, void* y, int
   launch_k(affine_fwd_x8_k, affine_blocks(n, C), 256, 0, st, (const bf16*)x, sc, sh, (bf16*)y, n / 8, C, relu);
 }
 void affine_add_x8(const void* x, const float* sc, const float* sh, const void* x2, const float* sc2,
-                   const float* sh2, void* y, int64_t n, int C, bool relu, cudaStream_t st) {
+                   const float* sh2, void* f, void* f2, void* y, int64_t n, int C, bool relu, cudaStream_t st) {
   launch_k(sc2 ? affine_add_x8_k<true> : affine_add_x8_k<false>, affine_blocks(n, C), 256, 0, st, (const bf16*)x, sc, sh,
-           (const bf16*)x2, sc2, sh2, (bf16*)y, n / 8, C, relu ? 1 : 0);
+           (const bf16*)x2, sc2, sh2, (bf16*)f, (bf16*)f2, (bf16*)y, n / 8, C, relu ? 1 : 0);
 }
 void affine_hswish_fwd_x8(const void* x, const float* sc, const float* sh, void* pre, void* post, int64_t n, int C,
                           cudaStream_t st) {
