@@ -128,9 +128,10 @@ typedef struct fo_server fo_server;
  * with fo_server_set_params.  Returns FO_ERR_UNSUPPORTED for layer shapes
  * without a kernel (e.g. bf16 conv channels not a multiple of 64), FO_ERR_ARG
  * for K or omega above FO_MAX_DEVICES / FO_MAX_OMEGA, for an op list whose
- * shapes do not chain, or for any tensor of more than 2^31 - 1 elements per
- * sample (all checked on the host before any CUDA call), FO_ERR_OOM when a
- * device or host allocation fails. */
+ * shapes do not chain, for any tensor of more than 2^31 - 1 elements per
+ * sample, or for a convolution or linear layer of about 2^31 pixels (rows) per
+ * batch or more (all checked on the host before any CUDA call), FO_ERR_OOM when
+ * a device or host allocation fails. */
 FO_API int fo_server_create(const fo_op* ops, int n_ops, const fo_optimizer* opt,
                      const fo_server_cfg* cfg, fo_server** out);
 FO_API int fo_server_destroy(fo_server* s);

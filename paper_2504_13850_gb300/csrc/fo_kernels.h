@@ -13,6 +13,10 @@ enum DType { kF32 = 0, kBF16 = 1 };
 struct ConvShape {
   int N, H, W, Ci, Co, k, stride, pad, Ho, Wo;
 };
+// Pixels and window elements are indexed in 32 bits, up to a tile or a rounded
+// K split (33 per split, two splits per SM) past the last one; server creation
+// refuses layers that do not leave this room.
+constexpr int64_t kIndexSlack = 65536;
 // y = conv(x, w) + bias, optional ReLU.  x NHWC, w [Co][k][k][Ci], bias fp32
 // or null, y NHWC; each operand's dtype is given (kF32 / kBF16).
 void conv_fwd_simt(const ConvShape& s, const void* x, int dt_x, const void* w, int dt_w,

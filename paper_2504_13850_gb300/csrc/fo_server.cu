@@ -170,6 +170,12 @@ int infer(fo_server* s) {
       default:
         return set_err(FO_ERR_ARG, "op " + std::to_string(i) + ": unknown kind");
     }
+    if (op.kind == FO_OP_CONV || op.kind == FO_OP_LINEAR) {
+      // the convolution kernels index pixels (linear layers: rows) and window elements in 32 bits
+      const int64_t kk = op.kind == FO_OP_CONV ? int64_t(op.k) * op.k : 1, most = INT32_MAX - fo::kIndexSlack;
+      if (a.rows() > most || kk * op.cin > most || kk * op.cout > most)
+        return set_err(FO_ERR_ARG, "op " + std::to_string(i) + ": more than 2^31 pixels per batch or window elements");
+    }
     if (int64_t(o.H) * o.W * o.C > INT32_MAX)
       return set_err(FO_ERR_ARG, "op " + std::to_string(i) + ": more than 2^31 - 1 elements per sample");
     s->T[i + 1] = o;

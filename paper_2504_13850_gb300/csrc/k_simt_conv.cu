@@ -9,9 +9,7 @@ namespace {
 
 Geo make_geo(const ConvShape& s, int mode) {
   Geo g{s.N, s.H, s.W, s.Ci, s.Co, s.k, s.stride, s.pad, s.Ho, s.Wo, 0, 0, 0, 1, 0};
-  // 32-bit pixel indices; more pixels than these give an empty grid, which the launch refuses
-  auto count = [](int64_t p) { return p > INT32_MAX - 4096 ? -1 : int(p); };
-  const int pix_out = count(int64_t(s.N) * s.Ho * s.Wo), pix_in = count(int64_t(s.N) * s.H * s.W);
+  const int pix_out = s.N * s.Ho * s.Wo, pix_in = s.N * s.H * s.W;   // within kIndexSlack of 2^31 (checked at creation)
   if (mode == FWD) {
     g.M = pix_out; g.Ncol = s.Co; g.K = s.k * s.k * s.Ci;
   } else if (mode == DGRAD) {

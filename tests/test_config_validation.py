@@ -63,6 +63,17 @@ def test_input_larger_than_int32_per_sample():
     refused("activation elements per sample", TINY, in_hwc=(65536, 65536, 1))
 
 
+@pytest.mark.parametrize("batch,hwc,ops,match", [
+    (1024, (2048, 2048, 1), [{"kind": "conv", "in0": 0, "cin": 1, "cout": 1, "k": 1, "stride": 2, "bias": 0}],
+     "pixels per batch"),
+    (512, (2048, 2048, 1), [{"kind": "linear", "in0": 0, "cin": 1, "cout": 1, "bias": 0}], "pixels per batch"),
+    (1, (1, 1, 240_000_000), [{"kind": "conv", "in0": 0, "cin": 240_000_000, "cout": 1, "k": 3, "stride": 1, "bias": 0}],
+     "window elements"),
+])
+def test_more_than_32_bits_of_pixels(batch, hwc, ops, match):
+    refused(match, TINY, batch=batch, in_hwc=hwc, ops=ops + head(1, 1))
+
+
 @pytest.mark.parametrize("ops,match", [
     ([{"kind": "relu", "in0": 1}] + head(1, 16 * 16 * 32), "bad in0"),
     ([{"kind": "conv", "in0": 0, "cin": 16, "cout": 8, "k": 3, "stride": 1, "bias": 0}] + head(1, 16 * 16 * 8),
