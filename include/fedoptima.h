@@ -254,7 +254,8 @@ FO_API int fo_set_device_active(fo_server* s, int device_id, int active);
 
 /* Bytes of the activation slab, omega slots of acts + labels + lengths: the
  * omega * mu_act term of Eq. 3, independent of K (a bf16 batch slot that a
- * convolution reads takes at least 128 KB).  -1 for a NULL handle.
+ * convolution reads through an im2col tensor map takes at least 128 KB).  -1
+ * for a NULL handle.
  * The helpers from here to fo_server_kernel_times have no counterpart in
  * the paper: they expose memory, streams and timing to the caller. */
 FO_API int64_t fo_server_activation_bytes(const fo_server* s);

@@ -1114,10 +1114,10 @@ int build_plan(fo_server* s) {
   return FO_OK;
 }
 
-// Bytes of a tensor's buffer: room for the images its im2col map declares.
+// Bytes of a buffer that an im2col map reads: room for the images it declares.
 int64_t im2col_room(const Tensor& t) {
   const int64_t image = int64_t(t.bytes()) / t.N;
-  return t.dt == fo::kBF16 ? fo::im2col_images(t.N, image) * image : int64_t(t.bytes());
+  return fo::im2col_images(t.N, image) * image;
 }
 
 int allocate(fo_server* s) {
@@ -1139,11 +1139,11 @@ int allocate(fo_server* s) {
   // activation slab: omega slots (Eq. 3), 256-byte aligned each
   s->slot_act_bytes = int64_t(c.batch) * c.in_h * c.in_w * c.in_c * esz;
   s->slot_stride = (s->slot_act_bytes + 255) / 256 * 256;
-  // a slot that a convolution window reads is long enough for its im2col map
-  if (s->dt == fo::kBF16)
-    for (const fo_op& op : s->ops)
-      if (op.kind == FO_OP_CONV && s->T[op.in0].is_input() && (op.k > 1 || op.stride > 1))
-        s->slot_stride = std::max(s->slot_stride, (im2col_room(s->T[0]) + 255) / 256 * 256);
+  // which activations and gradients im2col maps read (a view's through its root)
+  std::vector<char> act_im2col(s->ops.size() + 1, 0), grad_im2col(s->ops.size() + 1, 0);
+  for (int i = 0; i < int(s->ops.size()); ++i)
+    if (fo::tc_reads_im2col(s, i)) act_im2col[s->T[s->ops[i].in0].root] = grad_im2col[s->T[i + 1].root] = 1;
+  if (act_im2col[0]) s->slot_stride = std::max(s->slot_stride, (im2col_room(s->T[0]) + 255) / 256 * 256);
   s->slab = (char*)s->alloc(size_t(s->slot_stride) * c.omega);
   s->slot_labels = (int32_t*)s->alloc(size_t(c.omega) * c.batch * 4);
   s->slot_lengths = (int32_t*)s->alloc(size_t(c.omega) * c.batch * 4);
@@ -1172,14 +1172,13 @@ int allocate(fo_server* s) {
   for (int tid = 1; tid <= nops; ++tid) {
     Tensor& t = s->T[tid];
     if (t.root != tid) continue;
-    const size_t room = size_t(im2col_room(t));   // zero past the tensor
-    t.act = s->alloc(room);
-    t.grad = s->alloc(room);
+    const size_t act = act_im2col[tid] ? size_t(im2col_room(t)) : t.bytes();
+    const size_t grad = grad_im2col[tid] ? size_t(im2col_room(t)) : t.bytes();
+    t.act = s->alloc(act);
+    t.grad = s->alloc(grad);
     if (!t.act || !t.grad) return set_err(FO_ERR_OOM, "tensor allocation");
-    if (room > t.bytes()) {
-      FO_CUDA(cudaMemset(t.act, 0, room));
-      FO_CUDA(cudaMemset(t.grad, 0, room));
-    }
+    if (act > t.bytes()) FO_CUDA(cudaMemset(t.act, 0, act));   // zero past the tensor
+    if (grad > t.bytes()) FO_CUDA(cudaMemset(t.grad, 0, grad));
   }
   for (int tid = 1; tid <= nops; ++tid) {
     Tensor& t = s->T[tid];

@@ -15,14 +15,20 @@ namespace fo {
 struct TcContext;
 struct TcGemm;
 
-// im2col tensor maps never describe a tensor shorter than this: a shorter one
-// is declared with more images, so the buffers they read (activations and
-// their gradients, and batch slots) have room for these, zero past the tensor.
+// im2col tensor maps never describe a tensor shorter than this: for drivers up
+// to 13.1 CUTLASS corrects the encoded map of a tensor below 131,072 bytes, and
+// a map that is never that short needs no correction (what one does without it
+// was not tried).  A shorter tensor is declared with more images, so the buffers
+// that such maps read (tc_reads_im2col) have room for these, zero past the tensor.
 constexpr int64_t kIm2colMinBytes = 128 * 1024;
 inline int64_t im2col_images(int64_t n, int64_t image_bytes) {
   const int64_t least = (kIm2colMinBytes + image_bytes - 1) / image_bytes;
   return n > least ? n : least;
 }
+
+// True if a pass of convolution `op` reads its input and its output gradient
+// through im2col maps (shapes only; usable before tc_create).
+bool tc_reads_im2col(const fo_server* s, int op);
 
 int tc_create(TcContext** out, fo_server* s);
 void tc_destroy(TcContext* c);

@@ -218,8 +218,8 @@ bool window_ok(int H, int W, int rows_needed, int* rows, int* imgs) {
 // on the CUDA-core kernel before (bf16, 5-9 TFLOP/s against 200-240 here):
 // ResNet-18 stages 3-4 on 28 x 28 maps at batch 24, 20.6 -> 0.72 ms a step then;
 // the VGG part at batch 37, whose last tile is partial, 8.0 -> 0.26 ms.
-bool whole_windows(const fo_op& op, const Tensor& a, const Tensor& o) {
-  return op.stride == 1 || (a.H == 2 * o.H && a.W == 2 * o.W);
+bool tiled_windows(const fo_op& op, const Tensor& a, const Tensor& o, int pixels, int* rows, int* imgs) {
+  return (op.stride == 1 || (a.H == 2 * o.H && a.W == 2 * o.W)) && window_ok(o.H, o.W, pixels, rows, imgs);
 }
 
 
@@ -455,6 +455,14 @@ static void apply_epilogue(TcGemm* g, const TcEpilogue* ex) {
   }
 }
 
+bool tc_reads_im2col(const fo_server* s, int i) {
+  const fo_op& op = s->ops[i];
+  if (!bf16_server(s) || op.kind != FO_OP_CONV || plain_gemm(op) || op.cin % 64 || op.cout % 64) return false;
+  const Tensor &a = s->T[op.in0], &o = s->T[i + 1];
+  int rows, imgs;
+  return !tiled_windows(op, a, o, BM, &rows, &imgs) || !tiled_windows(op, a, o, BK, &rows, &imgs);
+}
+
 TcGemm* tc_plan_forward(TcContext* c, fo_server* s, int i, void* out, bool relu, const TcEpilogue* ex) {
   if (!c || !bf16_server(s) || getenv("FO_NO_TC")) return nullptr;
   const fo_op& op = s->ops[i];
@@ -496,7 +504,7 @@ TcGemm* tc_plan_forward(TcContext* c, fo_server* s, int i, void* out, bool relu,
   const int st = op.stride, Ho = o.H, Wo = o.W;
   if (op.cin % 64 || op.cout % 64) { delete g; return nullptr; }
   int rows, imgs;
-  const bool tiled = whole_windows(op, a, o) && window_ok(Ho, Wo, BM, &rows, &imgs);
+  const bool tiled = tiled_windows(op, a, o, BM, &rows, &imgs);
   if (ex && ex->pool_out && !tiled) { delete g; return nullptr; }
   g->kind = CONV_FPROP;
   g->name = "tc_conv_fprop";
@@ -563,7 +571,7 @@ bool tc_plan_dgrad(TcContext* c, fo_server* s, int i, int accumulate, void* dx, 
   const int st = op.stride, pad = op.k / 2, Ho = o.H, Wo = o.W;
   if (op.cin % 64 || op.cout % 64) return false;
   int rows, imgs;
-  const bool tiled = whole_windows(op, a, o) && window_ok(Ho, Wo, BM, &rows, &imgs);
+  const bool tiled = tiled_windows(op, a, o, BM, &rows, &imgs);
   const int nclass = st * st;
   bool any_empty = false;
   struct Cls { int n, H, W; int rs[9], dh[9], dw[9]; } cls[4];
@@ -671,7 +679,7 @@ TcGemm* tc_plan_wgrad(TcContext* c, fo_server* s, int i) {
   const int st = op.stride, Ho = o.H, Wo = o.W;
   if (op.cin % 64 || op.cout % 128) { delete g; return nullptr; }
   int rows, imgs;
-  const bool tiled = whole_windows(op, a, o) && window_ok(Ho, Wo, BK, &rows, &imgs);
+  const bool tiled = tiled_windows(op, a, o, BK, &rows, &imgs);
   g->kind = CONV_WGRAD;
   g->name = "tc_conv_wgrad";
   g->p.ldo = op.k * op.k * op.cin;
