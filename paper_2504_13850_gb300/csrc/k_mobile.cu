@@ -231,12 +231,15 @@ __device__ __forceinline__ void st8(bf16* p, const F8& r) {
   for (int j = 0; j < 8; ++j) e[j] = __float2bfloat16_rn(r.v[j]);
   *reinterpret_cast<uint4*>(p) = u;
 }
-__device__ __forceinline__ void fma8(F8& a, const F8& x, const float* w) {
-  const float4 w0 = *reinterpret_cast<const float4*>(w), w1 = *reinterpret_cast<const float4*>(w + 4);
-  a.v[0] = fmaf(x.v[0], w0.x, a.v[0]); a.v[1] = fmaf(x.v[1], w0.y, a.v[1]);
-  a.v[2] = fmaf(x.v[2], w0.z, a.v[2]); a.v[3] = fmaf(x.v[3], w0.w, a.v[3]);
-  a.v[4] = fmaf(x.v[4], w1.x, a.v[4]); a.v[5] = fmaf(x.v[5], w1.y, a.v[5]);
-  a.v[6] = fmaf(x.v[6], w1.z, a.v[6]); a.v[7] = fmaf(x.v[7], w1.w, a.v[7]);
+// a += x * w where `in`; else a as it is, also where w or x is not finite (a
+// zero in their place would give NaN).
+__device__ __forceinline__ void fma8(F8& a, const F8& x, const F8& w, bool in) {
+#pragma unroll
+  for (int j = 0; j < 8; ++j) a.v[j] = in ? fmaf(x.v[j], w.v[j], a.v[j]) : a.v[j];
+}
+__device__ __forceinline__ F8 ld8(const float* p) {
+  const float4 u = *reinterpret_cast<const float4*>(p), v = *reinterpret_cast<const float4*>(p + 4);
+  return {{u.x, u.y, u.z, u.w, v.x, v.y, v.z, v.w}};
 }
 
 // Block (channel block, pixel block of 16): DGRAD false, y = conv(x) + bias;
@@ -277,6 +280,7 @@ __global__ void __launch_bounds__(kDwThreads) dwconv_x8_k(const bf16* __restrict
       }
       hok = hok && h < Hx;
       uint4 u[KT];
+      bool in[KT];
 #pragma unroll
       for (int s = 0; s < KT; ++s) {
         int v = DGRAD ? j + d.pad - s : j * d.stride - d.pad + s;
@@ -286,11 +290,11 @@ __global__ void __launch_bounds__(kDwThreads) dwconv_x8_k(const bf16* __restrict
           v >>= 1;
         }
         ok = ok && v < Wx;
-        const uint4 t = *reinterpret_cast<const uint4*>(xn + (ok ? int64_t(h * Wx + v) * d.C : 0));
-        u[s] = ok ? t : make_uint4(0u, 0u, 0u, 0u);
+        u[s] = *reinterpret_cast<const uint4*>(xn + (ok ? int64_t(h * Wx + v) * d.C : 0));
+        in[s] = ok;
       }
 #pragma unroll
-      for (int s = 0; s < KT; ++s) fma8(a, up8(u[s]), &ws[r * KT + s][cv]);
+      for (int s = 0; s < KT; ++s) fma8(a, up8(u[s]), ld8(&ws[r * KT + s][cv]), in[s]);
     }
     bf16* out = y + int64_t(p) * d.C + c;
     if (acc_flag) {
@@ -336,19 +340,15 @@ __global__ void __launch_bounds__(240) dwconv_wgrad_x8_k(const bf16* __restrict_
       if (h < 0 || h >= d.H) continue;
       const bf16* xr = x + (n * d.H + h) * int64_t(d.W) * d.C + c;
       uint4 u[KT];
+      bool in[KT];
 #pragma unroll
       for (int s = 0; s < KT; ++s) {   // a tap outside the row loads its first pixel and drops it
         const int v = j * d.stride - d.pad + s;
-        const bool ok = v >= 0 && v < d.W;
-        const uint4 t = *reinterpret_cast<const uint4*>(xr + (ok ? int64_t(v) * d.C : 0));
-        u[s] = ok ? t : make_uint4(0u, 0u, 0u, 0u);
+        in[s] = v >= 0 && v < d.W;
+        u[s] = *reinterpret_cast<const uint4*>(xr + (in[s] ? int64_t(v) * d.C : 0));
       }
 #pragma unroll
-      for (int s = 0; s < KT; ++s) {
-        const F8 xv = up8(u[s]);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) a[s].v[q] = fmaf(dv.v[q], xv.v[q], a[s].v[q]);
-      }
+      for (int s = 0; s < KT; ++s) fma8(a[s], dv, up8(u[s]), in[s]);
     }
   float* mine = red + pl * (KK + 1) * (kDwC + 1) + cv;
 #pragma unroll
