@@ -730,15 +730,23 @@ __global__ void __launch_bounds__(256) finish_batch_k(const __grid_constant__ Fi
 
 int chunks_of(int64_t rows, int chunk) { return int((rows + chunk - 1) / chunk); }
 
-// Rows per chunk of the public column sums: the multiple of kChunk (so that the
-// partials fit what kChunk asks for) whose blocks run in one wave of eight per
-// SM.  Chunks of kChunk rows made 1.7 waves of 65,500 x 1000 and twice the
-// partials to finish (36.6 -> 34.2 us a call, with four rows in flight a thread).
+// Rows per chunk of the public column sums: the multiple of 8 whose blocks run
+// in one wave of as many as fit on every SM (six, at 40 registers a thread),
+// and no fewer than kChunk, so that the partials fit what kChunk asks for.
+// 65,500 x 1000, us a call: 36.4 in chunks of kChunk rows (1.7 waves of eight
+// rows in flight a block), 34.3 in multiples of kChunk for a wave of eight
+// blocks per SM, of which six fit, 26.1 here.  Eight blocks of 32 registers
+// (which spill) were slower on all but very long columns.
 int entry_chunk(int64_t rows, int C) {
-  const int64_t wave = 8 * int64_t(elementwise_blocks(int64_t(1) << 30, 256) / 8);   // eight blocks on every SM
+  static const int per_sm = [] {
+    int n = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, colsum8_k<0, 4>, 256, 0) != cudaSuccess) n = 0;
+    return n > 0 ? n : 4;
+  }();
+  const int64_t wave = per_sm * int64_t(elementwise_blocks(int64_t(1) << 30, 256) / 8);   // the cap there: 8 per SM
   const int64_t colblocks = (C + 255) / 256, most = std::max<int64_t>(1, wave / colblocks);
-  const int64_t m = (chunks_of(rows, kChunk) + most - 1) / most;
-  return int(m * kChunk);
+  const int64_t ch = ((rows + most - 1) / most + 7) / 8 * 8;
+  return int(std::max<int64_t>(ch, kChunk));
 }
 
 // Rows per chunk for the server's column sums: about two blocks per SM,
