@@ -261,15 +261,17 @@ int active_clusters(TcContext* c, int kind, int bn, int S, int epi) {
 //    issue of a stage, the 256-wide tile by 192 KB in flight over a TMA round
 //    trip of ~1.4 us.  In a step, narrow tiles cost the kernels beside them
 //    more L2 traffic for the same work; 0.30 / 0.32 / 0.375 gave the best
-//    whole steps (us; these / 0.37, 0.37, 0.375 / 0.21, 0.24, 0.36): VGG 270 /
-//    269 / 271, ResNet 540 / 544 / 532, ResNet on 28 x 28 maps 643 / 662 / 660,
-//    transformer 741 / 756 / 775, one narrow ragged block 269 / 278 / 289;
-//  * a launch that leaves SMs to others is charged the uncontended stage (0.21
-//    / 0.24 / 0.34): plain GEMMs on up to half of the SMs, tiled convolutions
-//    up to 0.85 of them, im2col windows never.  Whole steps with these limits
-//    at 0 / 0.5 / 0.85 for all kinds: ResNet 464 / 456 / 447, VGG 255 / 256 /
-//    253, one 384-wide encoder block 156 / 151 / 157, transformer 726 / 728 /
-//    755, ResNet on 28 x 28 maps 429 / 438 / 435;
+//    whole steps (us; these / 0.37, 0.37, 0.375 / the uncontended costs): VGG
+//    243 / 243 / 251, ResNet 436 / 434 / 447, on 28 x 28 maps 418 / 415 / 420,
+//    transformer 709 / 730 / 740, one narrow ragged block 129 / 125 / 126;
+//  * a launch that leaves SMs to others is charged nearer to the uncontended
+//    stage (0.21 / 0.24 / 0.34): convolutions on up to 0.85 of the SMs, plain
+//    GEMMs, more of which run side by side, on up to half.  Whole steps (us)
+//    with the convolutions' limit at 0 / 0.5 / 0.85: VGG 252 / 252 / 247, ResNet
+//    457 / 451 / 441, on 28 x 28 maps at batch 24 430 / 422 / 423, at batch 8
+//    303 / 295 / 290; with the plain GEMMs' at 0 / 0.5 / 0.85: transformer 718 /
+//    717 / 744, one 384-wide block 151 / 145 / 153, one 512-wide block of 40 x
+//    50 tokens 183 / 184 / 178;
 //  * a CTA pays a start-up ramp and the epilogue of its last tile (earlier
 //    epilogues overlap the next tile's MMAs), a K-split cluster pays the
 //    exchange of its partial tiles through the L2 workspace and their
@@ -293,7 +295,7 @@ void choose_tiles(TcContext* c, TcGemm* g, int M, int N, int KB, int ndiv) {
     const bool mn = g->kind == LIN_WGRAD || win_b;
     const double t_busy = (bn == 256 ? 0.375 : (bn == 128 ? 0.32 : 0.30)) + (mn ? 0.015 : 0.0);
     const double t_alone = (bn == 256 ? 0.34 : (bn == 128 ? 0.24 : 0.21)) + (mn ? 0.015 : 0.0);
-    const double alone = g->p.im2col ? 0.0 : (win_a || win_b ? 0.85 : 0.5);   // share of the SMs up to which it applies
+    const double alone = win_a || win_b ? 0.85 : 0.5;   // share of the SMs up to which it applies
     for (int sp = 1; sp <= 8; ++sp) {
       if (sp > 1 && KB / sp < 4) break;
       // an owner's receive slices (16 KB per other rank and owned chunk) live in the pipeline buffers
