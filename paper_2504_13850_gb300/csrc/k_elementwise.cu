@@ -472,7 +472,7 @@ __global__ void __launch_bounds__(256) avgpool_bwd_x8_k(const bf16* __restrict__
   }
 }
 void avgpool_fwd(const void* x, void* y, int N, int HW, int C, int dt, cudaStream_t st) {
-  if (dt == kBF16 && C % 8 == 0) {
+  if (dt == kBF16 && C % 8 == 0 && ceil_div(C, 256) <= 65535) {   // at most 256 channels per blockIdx.y
     int GL = 4;   // channel vectors per block: the fewest blocks' worth that covers C, at most a warp's
     while (GL < 32 && GL * 8 < C) GL *= 2;
     launch_k(avgpool_fwd_x8_k, dim3(N, ceil_div(C, GL * 8)), 256, 0, st, (const bf16*)x, (bf16*)y, HW, C, GL);

@@ -47,3 +47,25 @@ def test_block(c, two, swapped, relu, batch, h, w):
     _, _, recs = teacher_forced(cfg, ev)
     assert len(recs) == 4
     check_teacher_forced(recs)
+
+
+def test_more_channels_than_a_grid_dimension():
+    """One more block of 256 channels than a grid has rows: the scalar pool takes them."""
+    import numpy as np
+    c = 65535 * 256 + 8
+    b = W._Builder()
+    t = b.add("avgpool", 0)
+    t = b.add("linear", t, cin=c, cout=8, bias=0)
+    b.add("linear", t, cin=8, cout=3, bias=0)
+    s = api.Server(b.ops, 1, 1, 1, 1, (1, 1, c), 3, "bf16", 0.0, 0.0)
+    theta = np.zeros(s.n_params, np.float32)
+    theta[c - 1] = 1.0                  # the first layer's first output is the last channel
+    theta[8 * c] = 1.0                  # and the first logit is that
+    s.set_params(theta)
+    x = np.zeros((1, 1, 1, c), np.uint16)
+    x[..., -1] = 0x4000                 # 2.0
+    assert s.enqueue_activations(0, x, np.zeros(1, np.int32))[0] == api.OK
+    s.server_step()
+    loss = s.read_losses(0, 1)[0]
+    s.close()
+    assert abs(loss - np.log(np.exp(2.0) + 2.0) + 2.0) < 1e-5
