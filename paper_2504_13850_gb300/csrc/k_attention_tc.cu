@@ -21,8 +21,9 @@
 // not enough: 0.17-0.26% of the outputs and gradients differed from the exact
 // value rounded to bf16, against 0.01-0.04% on the fp32 CUDA-core kernels
 // that these widths ran on before.  A step of one 256-wide encoder block of
-// 19 x 77 tokens, 8 heads of 32: 289 us with those, 127 with two terms, 131
-// with three (64 x 128 tokens: 223 with two, 240 with three).
+// 19 x 77 tokens, 8 heads of 32: 289 us with those (and the GEMMs of then), 127
+// with two terms, 131 with three (64 x 128 tokens: 223 with two, 240 with
+// three).
 // Operand tiles are 128 rows x 64 bf16 (128-byte rows, 128-byte swizzle),
 // loaded by TMA from the packed q|k|v [B*L, 3C] and dO [B*L, C] (the
 // backward reads O's rows directly for rowsum(dO * O));

@@ -206,10 +206,9 @@ __global__ void __launch_bounds__(256) dwconv_wgrad_any_k(const T* __restrict__ 
 // a thread owns 8 channels (one 16-byte access per tap), a block 64 channels,
 // whose weights it stages once as fp32 [tap][channel].  The scalar kernels
 // above read a channel's k * k weights with a stride of k * k elements and
-// divide 64-bit indices per element, which bounded them.  Steps, us, scalar ->
-// here: MobileNet part on 4 x 4 maps at batch 64 417 -> 394; on 14 x 14 maps at
-// batch 32 (with the head's and the squeeze-and-excite block's changes)
-// 1498 -> 790.
+// divide 64-bit indices per element, which bounded them.  Steps, us, with the
+// scalar kernels and with these: MobileNet part on 4 x 4 maps at batch 64 372
+// and 350, on 14 x 14 maps at batch 32 1065 and 745.
 constexpr int kDwC = 64;        // channels per block
 constexpr int kDwV = kDwC / 8;  // threads over them
 

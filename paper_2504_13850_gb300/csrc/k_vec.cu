@@ -113,7 +113,7 @@ __global__ void grad_split_x8_k(const bf16* __restrict__ dy, const bf16* __restr
 // loads once: an index modulo in 64 bits and 16 scalar loads per vector cost
 // more than the traffic before.  With the residual adds below, ResNet stages
 // 3-4 at batch 128 went from 529 to 475 us a step, on 28 x 28 maps at batch 24
-// from 515 to 453.
+// from 515 to 453; the adds' share now is 446 -> 437 and 427 -> 418.
 __device__ __forceinline__ float round_bf16(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
 __device__ __forceinline__ float hswish_f(float v) { return v * fminf(fmaxf(v + 3.f, 0.f), 6.f) / 6.f; }
 __device__ __forceinline__ float hswish_d(float v) { return v < -3.f ? 0.f : (v > 3.f ? 1.f : (2.f * v + 3.f) / 6.f); }
@@ -472,8 +472,10 @@ __global__ void __launch_bounds__(256, 2) layernorm_fwd_x8_k(const bf16* __restr
 // connection passes around the layernorm.
 // Widths that are no multiple of 256, and 768 and 1024, ran as a scalar pass
 // and four column-sum launches before: a step of one encoder block at batch 16
-// x 100 tokens, us: 384 wide 222 -> 171, 768 wide 295 -> 239 (with the
-// classifier head's change).
+// x 100 tokens, us: 320 wide 167 -> 129, 384 wide 185 -> 144, 768 wide 262 ->
+// 213, 1024 wide 316 -> 263.  Which operands there are is a template parameter;
+// one variant spills, 22 bytes a thread: widths above 768 with both extra
+// operands and the partials of dx.
 constexpr int kLnWarps = 4;   // warps per block: the 4096-row step in 256 blocks
 constexpr int ln_rows_nv(int nv) { return nv <= 2 ? 4 : 2; }   // rows per warp: what its registers hold
 __device__ __forceinline__ float bf_at(const uint4& u, int j) {
