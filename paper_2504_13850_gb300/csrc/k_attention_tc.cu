@@ -22,7 +22,7 @@
 // value rounded to bf16, against 0.01-0.04% on the fp32 CUDA-core kernels
 // that these widths ran on before.  A step of one 256-wide encoder block of
 // 19 x 77 tokens, 8 heads of 32: 289 us with those (and the GEMMs of then), 127
-// with two terms, 131 with three (64 x 128 tokens: 223 with two, 240 with
+// with two terms, 130 with three (64 x 128 tokens: 223 with two, 237 with
 // three).
 // Operand tiles are 128 rows x 64 bf16 (128-byte rows, 128-byte swizzle),
 // loaded by TMA from the packed q|k|v [B*L, 3C] and dO [B*L, C] (the
@@ -75,8 +75,9 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
 __host__ __device__ constexpr uint32_t term_off(int t) { return t ? uint32_t(2 * t + 1) * kTile : 0u; }
 
 // v[0..8) as a sum of TERMS bf16 values, term t into the 16-byte unit at
-// at + term_off(t).  A term that overflows to infinity has no remainder.
-template <int TERMS>
+// at + term_off(t).  INF: values may be infinite (dS; P is at most 1), and a
+// term that is has no remainder.
+template <int TERMS, bool INF = false>
 __device__ __forceinline__ void st_unit(uint32_t at, float (&v)[8]) {
 #pragma unroll
   for (int t = 0; t < TERMS; ++t) {
@@ -86,8 +87,8 @@ __device__ __forceinline__ void st_unit(uint32_t at, float (&v)[8]) {
       h[q] = pack_bf16x2(v[2 * q], v[2 * q + 1]);
       if (t + 1 < TERMS) {
         const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&h[q]));
-        v[2 * q] = isinf(f.x) ? 0.f : v[2 * q] - f.x;
-        v[2 * q + 1] = isinf(f.y) ? 0.f : v[2 * q + 1] - f.y;
+        v[2 * q] = INF && isinf(f.x) ? 0.f : v[2 * q] - f.x;
+        v[2 * q + 1] = INF && isinf(f.y) ? 0.f : v[2 * q + 1] - f.y;
       }
     }
     st_shared4(at + term_off(t), h[0], h[1], h[2], h[3]);
@@ -465,7 +466,7 @@ __global__ void __launch_bounds__(kAttnThreads, SPLIT ? 1 : 2) attn_bwd_tc_k(con
         float v[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) v[e] = ds[8 * u + e];
-        st_unit<kTerms>(ds_base + hf * kTile + sw_off(i, u), v);
+        st_unit<kTerms, true>(ds_base + hf * kTile + sw_off(i, u), v);
       }
     } else {
 #pragma unroll 1
